@@ -9,6 +9,7 @@
 // and reversed in k; relu masks by a > 0. Adam (Kingma & Ba) with bias correction.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <memory>
@@ -23,95 +24,394 @@ namespace {
 
 #define TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) { set_last_cuda(e_); return e_ == cudaErrorMemoryAllocation ? VP_ERR_OOM : VP_ERR_CUDA; } } while (0)
 
-constexpr int kTX = 128;   // positions per block
-constexpr int kTO = 16;    // output channels per block
-constexpr int kTC = 8;     // input channels per shared chunk
 constexpr int kMaxK = 15;
+constexpr int kTC = 8;      // input channels per shared chunk
+constexpr int kTO = 64;     // output channels per block at most
+constexpr int kWPitch = kTO + 4;
 
-// out[b][o][x] = (bias ? bias[o] : 0) + sum_{c,k} w(o, c, k) in[b][c][(x + k - K/2) mod n]
-// with w(o, c, k) = W[o][c][k] (transpose = 0) or W[c][o][K-1-k] (transpose = 1, W of shape [Cin'][Cout'][K]).
-__global__ void __launch_bounds__(kTX) k_conv(int n, int Cin, int Cout, int K, int transpose, const float* __restrict__ W,
-                                             const float* __restrict__ bias, const float* __restrict__ in,
-                                             float* __restrict__ out, int relu) {
-  __shared__ float tile[kTC][kTX + kMaxK];
-  __shared__ float wsh[kTO][kTC][kMaxK];
-  const int x0 = blockIdx.x * kTX, o0 = blockIdx.y * kTO, b = blockIdx.z;
-  const int tx = threadIdx.x;
-  const int half = K / 2;
-  float acc[kTO];
-#pragma unroll
-  for (int o = 0; o < kTO; ++o) acc[o] = (bias && o0 + o < Cout) ? bias[o0 + o] : 0.f;
-  for (int c0 = 0; c0 < Cin; c0 += kTC) {
-    for (int e = tx; e < kTC * (kTX + K - 1); e += kTX) {
-      const int c = e / (kTX + K - 1), xx = e % (kTX + K - 1);
-      int gx = x0 + xx - half;
-      gx = ((gx % n) + n) % n;
-      tile[c][xx] = (c0 + c < Cin) ? in[((size_t)b * Cin + c0 + c) * n + gx] : 0.f;
-    }
-    for (int e = tx; e < kTO * kTC * K; e += kTX) {
-      const int o = e / (kTC * K), rem = e % (kTC * K), c = rem / K, k = rem % K;
-      float v = 0.f;
-      if (o0 + o < Cout && c0 + c < Cin) {
-        v = transpose ? W[((size_t)(c0 + c) * Cout + (o0 + o)) * K + (K - 1 - k)]
-                      : W[((size_t)(o0 + o) * Cin + (c0 + c)) * K + k];
-      }
-      wsh[o][c][k] = v;
-    }
-    __syncthreads();
-    if (x0 + tx < n) {
-      for (int c = 0; c < kTC; ++c)
-        for (int k = 0; k < K; ++k) {
-          const float v = tile[c][tx + k];
-#pragma unroll
-          for (int o = 0; o < kTO; ++o) acc[o] = fmaf(wsh[o][c][k], v, acc[o]);
-        }
-    }
-    __syncthreads();
-  }
-  if (x0 + tx < n) {
-#pragma unroll
-    for (int o = 0; o < kTO; ++o)
-      if (o0 + o < Cout) out[((size_t)b * Cout + o0 + o) * n + x0 + tx] = relu ? fmaxf(acc[o], 0.f) : acc[o];
-  }
+// Positions of halo kept on each side of a tile, a whole number of 16-byte groups.
+__host__ __device__ constexpr int halo(int K) { return (K / 2 + 3) / 4 * 4; }
+
+__device__ inline void cp_async16(float* smem, const float* gmem, bool valid) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  const int bytes = valid ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(bytes) : "memory");
+}
+__device__ inline void cp_async4(float* smem, const float* gmem, bool valid) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  const int bytes = valid ? 4 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sa), "l"(gmem), "r"(bytes) : "memory");
 }
 
-// dW[o][c][k] = sum_{b,x} dz[b][o][x] a[b][c][(x + k - K/2) mod n]; dbias[o] = sum dz (c == 0 blocks).
-__global__ void k_conv_wgrad(int n, int B, int Cin, int Cout, int K, const float* __restrict__ dz,
-                             const float* __restrict__ a, float* __restrict__ dW, float* __restrict__ dbias) {
-  const int o = blockIdx.x, c = blockIdx.y;
-  const int half = K / 2;
-  float s[kMaxK + 1];
-  for (int k = 0; k <= K; ++k) s[k] = 0.f;
-  for (int idx = threadIdx.x; idx < B * n; idx += blockDim.x) {
-    const int b = idx / n, x = idx % n;
-    const float g = dz[((size_t)b * Cout + o) * n + x];
-    const float* ar = a + ((size_t)b * Cin + c) * n;
-    for (int k = 0; k < K; ++k) {
-      int gx = x + k - half;
+// Rows r < rows of sm (pitch P) = src[r][(x0 + xx) mod n] for 0 <= xx < LEN (x0 >= -n), zeros for r >= have and for
+// x0 + xx >= lim. vec: src 16-byte aligned, n and x0 multiples of 4, so whole groups of 4 wrap together.
+template <int LEN, int P>
+__device__ inline void load_rows(float* sm, const float* src, int rows, int have, int n, int x0, int lim, bool vec,
+                                 int tid, int nt) {
+  static_assert(LEN % 4 == 0 && P % 4 == 0, "whole groups");
+  if (vec) {
+    for (int e = tid; e < rows * (LEN / 4); e += nt) {
+      const int r = e / (LEN / 4), x = (e - r * (LEN / 4)) * 4;
+      int gx = x0 + x;
+      const bool ok = r < have && gx < lim;
       gx = gx < 0 ? gx + n : (gx >= n ? gx - n : gx);
-      s[k] = fmaf(g, ar[gx], s[k]);
+      cp_async16(sm + r * P + x, ok ? src + (size_t)r * n + gx : src, ok);
     }
-    s[K] += g;
-  }
-  __shared__ float red[kMaxK + 1][32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int k = 0; k <= K; ++k) {
-    float v = s[k];
-    for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane == 0) red[k][wid] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x <= K) {
-    float v = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-    if (threadIdx.x < K) dW[((size_t)o * Cin + c) * K + threadIdx.x] = v;
-    else if (c == 0) dbias[o] = v;
+  } else {
+    for (int e = tid; e < rows * LEN; e += nt) {
+      const int r = e / LEN, x = e - r * LEN;
+      int gx = x0 + x;
+      const bool ok = r < have && gx < lim && gx >= -n;
+      gx = gx < 0 ? gx + n : (gx >= n ? gx - n : gx);
+      cp_async4(sm + r * P + x, ok ? src + (size_t)r * n + gx : src, ok);
+    }
   }
 }
 
-__global__ void k_relu_mask(size_t m, const float* __restrict__ a, float* __restrict__ g) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i < m && !(a[i] > 0.f)) g[i] = 0.f;
+__host__ __device__ inline int pad4(int c) { return (c + 3) & ~3; }
+
+// out[b][o][x] = (bias ? bias[o] : 0) + sum_{c,k} w(o, c, k) in[b][c][(x + k - K/2) mod n], the weights laid out as
+// W[c][k][pad4(Cout)] (k_layout); relu: max(., 0); mask (an array like out): 0 where mask is not positive.
+//
+// A thread holds OT output channels x XT groups of 4 positions in registers (the groups XG * 4 apart, so that
+// the 16-byte reads of the window are free of bank conflicts). Per input channel it reads the window of
+// K + 3 positions of each group once and, per tap, OT weights by broadcast: with 8 x 8 outputs and K = 9, 24
+// shared reads of 16 bytes for 576 multiply-adds, so the FP32 pipe bounds it and not shared memory (one
+// output per position read took 17 reads per 16 multiply-adds). Chunks of kTC channels are copied one ahead
+// by 16-byte cp.async (scalar loads of the parameter order cost as many instructions as the multiply-adds).
+// Every output is summed in the order of the definition, channel after channel, tap after tap.
+template <int K, int OT, int XT, int XG>
+__global__ void __launch_bounds__(256) k_conv(int n, int Cin, int Cout, const float* __restrict__ W,
+                                              const float* __restrict__ bias, const float* __restrict__ in,
+                                              float* __restrict__ out, int relu, const float* __restrict__ mask,
+                                              int vec) {
+  constexpr int TX = XG * 4 * XT, PAD = halo(K), TP = TX + 2 * PAD;  // positions of a block; row of the input tile
+  constexpr int half = K / 2, off = PAD - half;                    // first tap of a group's window
+  constexpr int NW = (off + K + 6) / 4;                            // 16-byte reads per window
+  extern __shared__ __align__(16) float conv_sm[];  // [2][input tile [kTC][TP], weights [kTC][K][kWPitch]]
+  constexpr int kBuf = kTC * (TP + K * kWPitch);
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int xg = tid % XG, og = tid / XG;
+  const int x0 = blockIdx.x * TX, o0 = blockIdx.y * kTO, b = blockIdx.z;
+  const int ldw = pad4(Cout), wq = min(kTO, ldw - o0) / 4;  // weight row; groups of 4 of it in this block
+  float acc[OT][XT][4];
+#pragma unroll
+  for (int r = 0; r < OT; ++r) {
+    const int o = o0 + og * OT + r;
+    const float v = (bias && o < Cout) ? bias[o] : 0.f;
+#pragma unroll
+    for (int j = 0; j < XT; ++j)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) acc[r][j][t] = v;
+  }
+  auto load = [&](int c0, float* sm) {
+    // positions past the last output's window are not used
+    load_rows<TP, TP>(sm, in + ((size_t)b * Cin + c0) * n, kTC, Cin - c0, n, x0 - PAD, n + half, vec, tid, nt);
+    float* ws = sm + kTC * TP;
+    const int rows = min(kTC, Cin - c0) * K;
+    for (int e = tid; e < kTC * K * wq; e += nt) {
+      const int row = e / wq, q = (e - row * wq) * 4;
+      const bool ok = row < rows;
+      cp_async16(ws + row * kWPitch + q, ok ? W + (size_t)(c0 * K + row) * ldw + o0 + q : W, ok);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  load(0, conv_sm);
+  for (int c0 = 0, st = 0; c0 < Cin; c0 += kTC, st ^= 1) {
+    if (c0 + kTC < Cin) {
+      load(c0 + kTC, conv_sm + (st ^ 1) * kBuf);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    }
+    __syncthreads();
+    const float* tile = conv_sm + st * kBuf;
+    const float* wsh = tile + kTC * TP;
+#pragma unroll 1
+    for (int c = 0; c < kTC; ++c) {
+      float win[XT][NW * 4];
+#pragma unroll
+      for (int j = 0; j < XT; ++j)
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+          const float4 v = *reinterpret_cast<const float4*>(tile + c * TP + (j * XG + xg + q) * 4);
+          win[j][4 * q] = v.x; win[j][4 * q + 1] = v.y; win[j][4 * q + 2] = v.z; win[j][4 * q + 3] = v.w;
+        }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        float w[OT];
+        if constexpr (OT >= 4) {
+#pragma unroll
+          for (int r = 0; r < OT; r += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(wsh + (c * K + k) * kWPitch + og * OT + r);
+            w[r] = v.x; w[r + 1] = v.y; w[r + 2] = v.z; w[r + 3] = v.w;
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < OT; ++r) w[r] = wsh[(c * K + k) * kWPitch + og * OT + r];
+        }
+#pragma unroll
+        for (int r = 0; r < OT; ++r)
+#pragma unroll
+          for (int j = 0; j < XT; ++j)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) acc[r][j][t] = fmaf(w[r], win[j][off + k + t], acc[r][j][t]);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int r = 0; r < OT; ++r) {
+    const int o = o0 + og * OT + r;
+    if (o >= Cout) break;
+    float* y = out + ((size_t)b * Cout + o) * n;
+    const float* m = mask ? mask + ((size_t)b * Cout + o) * n : nullptr;
+#pragma unroll
+    for (int j = 0; j < XT; ++j) {
+      const int x = x0 + (j * XG + xg) * 4;
+      float v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        v[t] = relu ? fmaxf(acc[r][j][t], 0.f) : acc[r][j][t];
+        if (m && x + t < n && !(m[x + t] > 0.f)) v[t] = 0.f;
+      }
+      if (vec) {
+        if (x < n) *reinterpret_cast<float4*>(y + x) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+          if (x + t < n) y[x + t] = v[t];
+      }
+    }
+  }
+}
+
+template <int K, int XT, int XG>
+constexpr size_t conv_smem() { return (size_t)2 * kTC * (XG * 4 * XT + 2 * halo(K) + K * kWPitch) * sizeof(float); }
+
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+template <int K, int OT, int XT, int XG>
+int launch_conv(int n, int B, int Cin, int Cout, const float* W, const float* bias, const float* in, float* out,
+                int relu, const float* mask, cudaStream_t s) {
+  constexpr int TX = XG * 4 * XT;
+  const int co = std::min(Cout, kTO), vec = n % 4 == 0 && aligned16(in) && aligned16(out);
+  k_conv<K, OT, XT, XG><<<dim3((n + TX - 1) / TX, (Cout + kTO - 1) / kTO, B), (co + OT - 1) / OT * XG,
+                          conv_smem<K, XT, XG>(), s>>>(n, Cin, Cout, W, bias, in, out, relu, mask, vec);
+  TRY(cudaGetLastError());
+  return VP_OK;
+}
+
+// 8 x 8 outputs a thread where that gives every SM two blocks (304 on 152 SMs); 4 x 4 where it does not (four
+// times the threads); one output channel a thread for at most two of them, which would leave most of an 8 x 8
+// tile empty. Measured (64 -> 64 channels, K = 9, n = 4096): batch 32 204 us = 47 TFLOP/s, FP32 pipe 67 % busy (389 us
+// with one position per thread); batch 1, 4 x 4 tiles, the whole network of four layers 66 us (243).
+template <int K>
+int launch_conv_k(int n, int B, int Cin, int Cout, const float* W, const float* bias, const float* in, float* out,
+                  int relu, const float* mask, cudaStream_t s) {
+  const long long blocks = (long long)((n + 127) / 128) * ((Cout + kTO - 1) / kTO) * B;
+  const auto f = Cout <= 2 ? launch_conv<K, 1, 1, 16> : (blocks >= 304 ? launch_conv<K, 8, 2, 16> : launch_conv<K, 4, 1, 8>);
+  return f(n, B, Cin, Cout, W, bias, in, out, relu, mask, s);
+}
+
+// The weights of a layer ([out][in][k] in p) as k_conv reads them: wf[in][k][pad4(out)] for the forward pass, and
+// wb[out][k][pad4(in)], reversed in k, for the transposed convolution of the backward pass. The padding is zero from
+// the allocation on.
+__global__ void k_layout(int Cin, int Cout, int K, const float* __restrict__ p, float* __restrict__ wf,
+                         float* __restrict__ wb) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= Cin * Cout * K) return;
+  const int o = e / (Cin * K), rem = e - o * Cin * K, c = rem / K, k = rem - c * K;
+  const float v = p[e];
+  wf[(size_t)(c * K + k) * pad4(Cout) + o] = v;
+  wb[(size_t)(o * K + K - 1 - k) * pad4(Cin) + c] = v;
+}
+
+// Part sums of dW[o][c][k] = sum_{b,x} dz[b][o][x] a[b][c][(x + k - K/2) mod n] and dbias[o] = sum dz over a
+// segment of the positions: block (seg, o tile, c tile) takes every gridDim.x-th chunk of kWX positions.
+// A thread holds OT output channels x 2 input channels x K taps in registers and walks along x four positions at a
+// time, so an input position is read once for its K taps: with OT = 4 and K = 9, 10 shared reads of 16 bytes for
+// 288 multiply-adds (one (o, c) pair per block read 10 values from L1 per 10 multiply-adds). Chunks are copied
+// to shared memory one ahead (cp.async). Row pitches of 4 mod 32 words and channels dealt out row by row keep
+// the reads free of bank conflicts. part[seg][Cout Cin K + Cout] is summed by k_sum_parts, so the result does
+// not depend on the order in which blocks run.
+// Measured (64 x 64 channels, K = 9, n = 4096, batch 32): 227 us = 43 TFLOP/s, FP32 pipe 58 % busy, 13 us for the
+// sum (about 3.3 ms with a block per (o, c) pair).
+constexpr int kWX = 64;                   // positions per chunk
+constexpr int kWPitchZ = kWX + 4;         // row of the dz chunk
+constexpr int kWPitchA = kWX + 20;        // row of the activation chunk (halos of at most 8 on each side)
+
+template <int K, int OT>
+__global__ void __launch_bounds__(512) k_conv_wgrad(int n, int B, int Cin, int Cout, const float* __restrict__ dz,
+                                                    const float* __restrict__ a, float* __restrict__ part,
+                                                    size_t part_ld, int vec) {
+  extern __shared__ __align__(16) float wg_sm[];
+  constexpr int half = K / 2, PAD = halo(K), off = PAD - half, NW = (off + K + 6) / 4;
+  constexpr int kOTile = 16 * OT;
+  const int o0 = blockIdx.y * kOTile, c0 = blockIdx.z * kTO;
+  const int no = min(kOTile, Cout - o0), nc = min(kTO, Cin - c0);
+  const int nog = (no + OT - 1) / OT, ncg = (nc + 1) / 2;
+  const int zrows = nog * OT, arows = ncg * 2;
+  const int buf = zrows * kWPitchZ + arows * kWPitchA;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int cg = tid % ncg, og = tid / ncg;
+  const bool live = og < nog;
+  const int nx = (n + kWX - 1) / kWX, chunks = B * nx;
+
+  auto load = [&](int ch, float* sm) {
+    const int b = ch / nx, x0 = (ch - b * nx) * kWX;
+    load_rows<kWX, kWPitchZ>(sm, dz + ((size_t)b * Cout + o0) * n, zrows, no, n, x0, n, vec, tid, nt);
+    load_rows<kWX + 2 * PAD, kWPitchA>(sm + zrows * kWPitchZ, a + ((size_t)b * Cin + c0) * n, arows, nc, n, x0 - PAD,
+                                      n + half, vec, tid, nt);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+
+  float acc[OT][2][K];
+#pragma unroll
+  for (int r = 0; r < OT; ++r)
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int k = 0; k < K; ++k) acc[r][q][k] = 0.f;
+  float bsum = 0.f;
+  int ch = blockIdx.x, st = 0;
+  if (ch < chunks) load(ch, wg_sm);
+  for (; ch < chunks; ch += gridDim.x, st ^= 1) {
+    const int next = ch + gridDim.x;
+    if (next < chunks) {
+      load(next, wg_sm + (st ^ 1) * buf);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    }
+    __syncthreads();
+    const float* sz = wg_sm + st * buf;
+    const float* sa = sz + zrows * kWPitchZ;
+    if (live) {
+#pragma unroll 1
+      for (int x = 0; x < kWX; x += 4) {
+        float d[OT][4], w[2][NW * 4];
+#pragma unroll
+        for (int r = 0; r < OT; ++r) {
+          const float4 v = *reinterpret_cast<const float4*>(sz + (og + r * nog) * kWPitchZ + x);
+          d[r][0] = v.x; d[r][1] = v.y; d[r][2] = v.z; d[r][3] = v.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+          for (int t = 0; t < NW; ++t) {
+            const float4 v = *reinterpret_cast<const float4*>(sa + (cg + q * ncg) * kWPitchA + x + 4 * t);
+            w[q][4 * t] = v.x; w[q][4 * t + 1] = v.y; w[q][4 * t + 2] = v.z; w[q][4 * t + 3] = v.w;
+          }
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int r = 0; r < OT; ++r)
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+              for (int k = 0; k < K; ++k) acc[r][q][k] = fmaf(d[r][t], w[q][off + t + k], acc[r][q][k]);
+      }
+    }
+    if (blockIdx.z == 0 && tid < no) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int x = 0; x < kWX; x += 4) {
+        const float4 z = *reinterpret_cast<const float4*>(sz + tid * kWPitchZ + x);
+        v.x += z.x; v.y += z.y; v.z += z.z; v.w += z.w;
+      }
+      bsum += (v.x + v.y) + (v.z + v.w);
+    }
+    __syncthreads();
+  }
+  float* pw = part + (size_t)blockIdx.x * part_ld;
+  if (live) {
+#pragma unroll
+    for (int r = 0; r < OT; ++r)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int o = og + r * nog, c = cg + q * ncg;
+        if (o < no && c < nc)
+#pragma unroll
+          for (int k = 0; k < K; ++k) pw[((size_t)(o0 + o) * Cin + c0 + c) * K + k] = acc[r][q][k];
+      }
+  }
+  if (blockIdx.z == 0 && tid < no) pw[(size_t)Cout * Cin * K + o0 + tid] = bsum;
+}
+
+size_t wgrad_smem(int zrows, int arows) { return (size_t)2 * (zrows * kWPitchZ + arows * kWPitchA) * sizeof(float); }
+
+template <int K>
+int launch_wgrad_k(int n, int B, int Cin, int Cout, const float* dz, const float* a, float* part, int segs,
+                   cudaStream_t s) {
+  constexpr int OT = K <= 9 ? 4 : 2, kOTile = 16 * OT;  // at most 72 sums per thread
+  const int no = std::min(Cout, kOTile), nc = std::min(Cin, kTO);
+  const int nog = (no + OT - 1) / OT, ncg = (nc + 1) / 2;
+  const int threads = std::max(64, (nog * ncg + 31) / 32 * 32);  // a thread per output channel for the bias sums
+  k_conv_wgrad<K, OT><<<dim3(segs, (Cout + kOTile - 1) / kOTile, (Cin + kTO - 1) / kTO), threads,
+                        wgrad_smem(nog * OT, ncg * 2), s>>>(n, B, Cin, Cout, dz, a, part,
+                                                            (size_t)Cout * Cin * K + Cout,
+                                                            n % 4 == 0 && aligned16(dz) && aligned16(a));
+  TRY(cudaGetLastError());
+  return VP_OK;
+}
+
+template <int K>
+int prepare_k() {
+  TRY(cudaFuncSetAttribute(k_conv_wgrad<K, (K <= 9 ? 4 : 2)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)wgrad_smem(kTO, kTO)));
+  TRY(cudaFuncSetAttribute(k_conv<K, 1, 1, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem<K, 1, 16>()));
+  TRY(cudaFuncSetAttribute(k_conv<K, 8, 2, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem<K, 2, 16>()));
+  TRY(cudaFuncSetAttribute(k_conv<K, 4, 1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem<K, 1, 8>()));
+  return VP_OK;
+}
+
+// Kernel sizes are odd and at most kMaxK.
+#define WS_BY_K(k, call)                 \
+  switch (k) {                           \
+    case 1: return call<1>;              \
+    case 3: return call<3>;              \
+    case 5: return call<5>;              \
+    case 7: return call<7>;              \
+    case 9: return call<9>;              \
+    case 11: return call<11>;            \
+    case 13: return call<13>;            \
+    default: return call<15>;            \
+  }
+auto conv_of(int k) -> decltype(&launch_conv_k<1>) { WS_BY_K(k, launch_conv_k) }
+auto wgrad_of(int k) -> decltype(&launch_wgrad_k<1>) { WS_BY_K(k, launch_wgrad_k) }
+auto prepare_of(int k) -> decltype(&prepare_k<1>) { WS_BY_K(k, prepare_k) }
+
+// Segments of a weight gradient: two blocks per SM of the 152 for the widest layers (an uneven last wave costs
+// less, and the running sums are half as long as with one), as far as the part sums fit kPartBytes.
+constexpr int kMaxSegs = 304;
+constexpr size_t kPartBytes = (size_t)128 << 20;
+int wgrad_segs(size_t layer_params) {
+  return (int)std::max<size_t>(1, std::min<size_t>(kMaxSegs, kPartBytes / (layer_params * sizeof(float))));
+}
+
+// g[p] = sum over the segments of part[seg][p], compensated: 32 parameters per block, warp w taking the
+// segments w mod 8, the eight sums added in their order.
+__global__ void __launch_bounds__(256) k_sum_parts(int m, int segs, const float* __restrict__ part, float* __restrict__ g) {
+  __shared__ float2 sh[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+  float s = 0.f, e = 0.f;
+  auto add = [&](float v) {
+    const float t = s + v, bb = t - s;
+    e += (s - (t - bb)) + (v - bb);
+    s = t;
+  };
+  if (p < m) {
+#pragma unroll 8
+    for (int q = w; q < segs; q += 8) add(part[(size_t)q * m + p]);
+  }
+  sh[w][lane] = make_float2(s, e);
+  __syncthreads();
+  if (w || p >= m) return;
+  for (int q = 1; q < 8; ++q) {
+    add(sh[q][lane].x);
+    e += sh[q][lane].y;
+  }
+  g[p] = s + e;
 }
 
 // g = 2 (y - t) / m and partial sums of (y - t)^2 (one per block, into part[blockIdx.x]).
@@ -155,9 +455,11 @@ struct ws_s {
   std::vector<size_t> woff, boff;           // parameter offsets
   size_t nparams = 0;
   float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
+  std::vector<float*> wf, wb;               // per layer: the weights as k_conv reads them (k_layout)
   std::vector<float*> act;                  // activations a_0..a_{L-1}, z_L (size L+1), max_batch each
   float *d0 = nullptr, *d1 = nullptr;       // gradient work buffers
   double* part = nullptr;
+  float* wparts = nullptr;                  // part sums of one layer's weight gradient
   long long step = 0;
   std::vector<void*> allocs;
 };
@@ -182,15 +484,25 @@ inline uint64_t splitmix64(uint64_t& s) {
   return z ^ (z >> 31);
 }
 
-int forward(ws_s* w, const float* x, int B, cudaStream_t s) {
-  const float* in = x;
+// The convolution layouts of the weights, after every change of the parameters.
+int layout(ws_s* w, cudaStream_t s) {
   for (int l = 0; l < w->L; ++l) {
     const int Cin = w->C[l], Cout = w->C[l + 1];
-    float* out = w->act[l + 1];
-    dim3 grid((w->n + kTX - 1) / kTX, (Cout + kTO - 1) / kTO, B);
-    k_conv<<<grid, kTX, 0, s>>>(w->n, Cin, Cout, w->K, 0, w->p + w->woff[l], w->p + w->boff[l], in, out,
-                                l < w->L - 1 ? 1 : 0);
+    k_layout<<<(unsigned)(((size_t)Cin * Cout * w->K + 255) / 256), 256, 0, s>>>(Cin, Cout, w->K, w->p + w->woff[l],
+                                                                              w->wf[l], w->wb[l]);
     TRY(cudaGetLastError());
+  }
+  return VP_OK;
+}
+
+// y: destination of the last layer.
+int forward(ws_s* w, const float* x, int B, float* y, cudaStream_t s) {
+  const float* in = x;
+  for (int l = 0; l < w->L; ++l) {
+    float* out = l == w->L - 1 ? y : w->act[l + 1];
+    const int rc = conv_of(w->K)(w->n, B, w->C[l], w->C[l + 1], w->wf[l], w->p + w->boff[l], in, out,
+                                 l < w->L - 1 ? 1 : 0, nullptr, s);
+    if (rc) return rc;
     in = out;
   }
   return VP_OK;
@@ -199,7 +511,7 @@ int forward(ws_s* w, const float* x, int B, cudaStream_t s) {
 int grad(ws_s* w, const float* x, const float* t, int B, float* loss, cudaStream_t s) {
   if (B < 1 || B > w->max_batch) return VP_ERR_ARG;
   // keep the input as a_0 (read only; the caller's buffer)
-  int rc = forward(w, x, B, s);
+  int rc = forward(w, x, B, w->act[w->L], s);
   if (rc) return rc;
   const size_t mout = (size_t)B * w->out_ch * w->n;
   const int nb = 256;
@@ -210,15 +522,14 @@ int grad(ws_s* w, const float* x, const float* t, int B, float* loss, cudaStream
   for (int l = w->L - 1; l >= 0; --l) {
     const int Cin = w->C[l], Cout = w->C[l + 1];
     const float* a = (l == 0) ? x : w->act[l];
-    k_conv_wgrad<<<dim3(Cout, Cin), 256, 0, s>>>(w->n, B, Cin, Cout, w->K, dz, a, w->g + w->woff[l],
-                                                 w->g + w->boff[l]);
+    const size_t m = (size_t)Cout * Cin * w->K + Cout;  // weights, then bias
+    const int segs = wgrad_segs(m);
+    if ((rc = wgrad_of(w->K)(w->n, B, Cin, Cout, dz, a, w->wparts, segs, s))) return rc;
+    k_sum_parts<<<(unsigned)((m + 31) / 32), 256, 0, s>>>((int)m, segs, w->wparts, w->g + w->woff[l]);
     TRY(cudaGetLastError());
     if (l > 0) {
-      dim3 grid((w->n + kTX - 1) / kTX, (Cin + kTO - 1) / kTO, B);
-      k_conv<<<grid, kTX, 0, s>>>(w->n, Cout, Cin, w->K, 1, w->p + w->woff[l], nullptr, dz, da, 0);
-      const size_t ma = (size_t)B * Cin * w->n;
-      k_relu_mask<<<(unsigned)((ma + 255) / 256), 256, 0, s>>>(ma, w->act[l], da);
-      TRY(cudaGetLastError());
+      // da masked by the activation of the layer
+      if ((rc = conv_of(w->K)(w->n, B, Cout, Cin, w->wb[l], nullptr, dz, da, 0, w->act[l], s))) return rc;
       std::swap(dz, da);
     }
   }
@@ -275,6 +586,19 @@ extern "C" int ws_create(int in_ch, int width, int out_ch, int n_layers, int ksi
   if ((rc = walloc(w.get(), &w->d0, (size_t)max_batch * maxc * n)) ||
       (rc = walloc(w.get(), &w->d1, (size_t)max_batch * maxc * n)))
     return fail(rc);
+  size_t parts = 0;
+  w->wf.assign(n_layers, nullptr);
+  w->wb.assign(n_layers, nullptr);
+  for (int l = 0; l < n_layers; ++l) {
+    const size_t nf = (size_t)w->C[l] * ksize * pad4(w->C[l + 1]), nb = (size_t)w->C[l + 1] * ksize * pad4(w->C[l]);
+    if ((rc = walloc(w.get(), &w->wf[l], nf)) || (rc = walloc(w.get(), &w->wb[l], nb))) return fail(rc);
+    if (cudaMemsetAsync(w->wf[l], 0, nf * sizeof(float), s) != cudaSuccess ||
+        cudaMemsetAsync(w->wb[l], 0, nb * sizeof(float), s) != cudaSuccess)
+      return fail(VP_ERR_CUDA);
+    const size_t m = (size_t)w->C[l + 1] * w->C[l] * ksize + w->C[l + 1];
+    parts = std::max(parts, m * wgrad_segs(m));
+  }
+  if ((rc = walloc(w.get(), &w->wparts, parts)) || (rc = prepare_of(ksize)())) return fail(rc);
   {
     void* q = nullptr;
     if (cudaMalloc(&q, 256 * sizeof(double)) != cudaSuccess) return fail(VP_ERR_OOM);
@@ -292,7 +616,7 @@ extern "C" int ws_create(int in_ch, int width, int out_ch, int n_layers, int ksi
     }
   }
   if (cudaMemcpyAsync(w->p, host.data(), off * sizeof(float), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemsetAsync(w->m, 0, off * sizeof(float), s) != cudaSuccess ||
+      layout(w.get(), s) != VP_OK || cudaMemsetAsync(w->m, 0, off * sizeof(float), s) != cudaSuccess ||
       cudaMemsetAsync(w->v, 0, off * sizeof(float), s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
     return fail(VP_ERR_CUDA);
   *out = w.release();
@@ -310,16 +634,17 @@ extern "C" int ws_params(ws_net net, float* buf, int get, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (get) TRY(cudaMemcpyAsync(buf, net->p, net->nparams * sizeof(float), cudaMemcpyDeviceToDevice, s));
   else TRY(cudaMemcpyAsync(net->p, buf, net->nparams * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  return VP_OK;
+  return get ? VP_OK : layout(net, s);
 }
 
 extern "C" int ws_forward(ws_net net, const float* x, int batch, float* y, void* stream) {
   if (!net || !x || !y || batch < 1 || batch > net->max_batch) return VP_ERR_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int rc = forward(net, x, batch, s);
+  // a single layer reads x while it writes: it goes through the activation buffer, so y may be x as before
+  if (net->L > 1) return forward(net, x, batch, y, s);
+  const int rc = forward(net, x, batch, net->act[1], s);
   if (rc) return rc;
-  TRY(cudaMemcpyAsync(y, net->act[net->L], (size_t)batch * net->out_ch * net->n * sizeof(float),
-                      cudaMemcpyDeviceToDevice, s));
+  TRY(cudaMemcpyAsync(y, net->act[1], (size_t)batch * net->out_ch * net->n * sizeof(float), cudaMemcpyDeviceToDevice, s));
   return VP_OK;
 }
 
@@ -344,5 +669,5 @@ extern "C" int ws_train_step(ws_net net, const float* x, const float* t, int bat
   k_adam<<<(unsigned)((net->nparams + 255) / 256), 256, 0, s>>>(net->nparams, net->p, net->g, net->m, net->v, lr, b1,
                                                                  b2, 1e-8f, c1, c2);
   TRY(cudaGetLastError());
-  return VP_OK;
+  return layout(net, s);
 }
