@@ -51,75 +51,154 @@ struct GemmArgs {
   const long long* dst_off;
 };
 
-// FP64 gather-GEMM: tile (64 rows x 64 columns), K in steps of 16, 256 threads,
-// each thread 4 rows (strided by 16) x 4 columns; rows of a destination vector
-// are contiguous, so a half-warp stores 16 consecutive doubles.
-constexpr int kBM = 64, kBN = 64, kBK = 16;
+// FP64 gather-GEMM on tiles of 32 rows x 32 columns, K in steps of 16 staged one ahead (cp.async), 128 threads: warp
+// w has columns 8 w .. 8 w + 7, lane (tr, cl) rows tr + 8 i (i < 4) and columns 8 w + cl + 4 j (j < 2).
+//
+// The FP64 pipe (2 multiply-adds per clock and SM) bounds it; operands are cheap beside that, so tiles are as
+// small as they need to be for little work on padding: rows are skipped in groups of 8 and columns in groups of 4
+// past the tile's own, and K ends where it ends (81-row operators run 88 of them, not 128, and groups of a few
+// columns only those). Measured (583-leaf adaptive tree, p = 16, both channels): near launch 3,343 -> 1,720 us =
+// 1.14 TFLOP/s, 0.91 of the pipe; M2L 973 -> 416 us (64 x 64 tiles computed whole).
+constexpr int kBM = 32, kBN = 32, kBK = 16, kGemmThreads = 128;
+// Launches of fewer tiles (16 per SM of the 152) leave SMs idle or uneven: they run on tiles of 8 x 4
+// (k_gemm_small_f64). Measured with the line at 608, 1216 and 2432 tiles: uniform depth 4, p = 11, 355, 311 and 311 us;
+// 60,000 nodes, p = 8, 702, 703 and 667 us; larger trees within 0.4 %.
+constexpr int kBMs = 8, kBNs = 4, kSmallTiles = 2432;
 
 // Deepest leaf level vp_tree_interp serves (its cell map holds 4^L ints: 256 MB at L = 13).
 constexpr int kInterpMaxLevel = 13;
 
+__device__ inline void cp_async8(double* smem, const double* gmem, bool valid) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  const int bytes = valid ? 8 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gmem), "r"(bytes) : "memory");
+}
+
+template <int RG, int CG>
+__device__ inline void fma_step(const double (*As)[kBM + 2], const double (*Bs)[kBN + 2], int kn, int tr, int cb,
+                                double (&acc)[4][2]) {
+#pragma unroll 4
+  for (int kk = 0; kk < kn; ++kk) {
+    double av[RG], bv[CG];
+#pragma unroll
+    for (int i = 0; i < RG; ++i) av[i] = As[kk][tr + 8 * i];
+#pragma unroll
+    for (int j = 0; j < CG; ++j) bv[j] = Bs[kk][cb + 4 * j];
+#pragma unroll
+    for (int i = 0; i < RG; ++i)
+#pragma unroll
+      for (int j = 0; j < CG; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+  }
+}
+
 // TAG only names the instantiation (1: near-field tables) so profilers can pick it out.
 template <int TAG>
-__global__ void __launch_bounds__(256) k_gemm_gather_f64(GemmArgs a) {
-  __shared__ double As[kBK][kBM + 2];
-  __shared__ double Bs[kBK][kBN + 2];
+__global__ void __launch_bounds__(kGemmThreads) k_gemm_gather_f64(GemmArgs a) {
+  __shared__ __align__(16) double As[2][kBK][kBM + 2];
+  __shared__ __align__(16) double Bs[2][kBK][kBN + 2];
   const Tile tile = a.tiles[blockIdx.x];
   const double* __restrict__ A = a.A + a.a_off[tile.group];
-  const int tid = threadIdx.x;
-  const int tr = tid & 15;   // row lane
-  const int tc = tid >> 4;   // column group (0..15)
-  double acc[4][4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tr = lane & 7, cb = warp * 8 + (lane >> 3);
+  const int rg = min(4, (a.M - tile.m0 + 7) / 8);                        // row groups of 8 in the tile
+  const int cg = max(0, min(2, (tile.ncol - warp * 8 + 3) / 4));          // column groups of 4 of this warp
+  // staging: thread (kk, r0) copies k = kk of rows and columns r0, r0 + 8, r0 + 16, r0 + 24
+  const int kk = tid & (kBK - 1), r0 = tid / kBK;
+  long long src[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) src[i] = r0 + 8 * i < tile.ncol ? a.src_off[tile.col0 + r0 + 8 * i] : -1;
+  auto load = [&](int st, int k0) {
+    const int gk = k0 + kk, sg = gk / a.kseg, off = gk - sg * a.kseg;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = r0 + 8 * i, gm = tile.m0 + r;
+      const bool ra = gm < a.M && gk < a.K, rb = src[i] >= 0 && gk < a.K;
+      cp_async8(&As[st][kk][r], ra ? A + (size_t)gm * a.lda + gk : A, ra);
+      cp_async8(&Bs[st][kk][r], rb ? a.X + src[i] + sg * a.seg_stride + off : a.X, rb);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  double acc[4][2];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-
-  for (int k0 = 0; k0 < a.K; k0 += kBK) {
-    // A tile: 64 rows x 16 k
-    for (int e = tid; e < kBM * kBK; e += 256) {
-      const int r = e / kBK, kk = e % kBK;
-      const int gm = tile.m0 + r, gk = k0 + kk;
-      As[kk][r] = (gm < a.M && gk < a.K) ? A[(size_t)gm * a.lda + gk] : 0.0;
-    }
-    // B tile: 16 k x 64 columns, gathered
-    for (int e = tid; e < kBN * kBK; e += 256) {
-      const int c = e / kBK, kk = e % kBK;
-      const int gk = k0 + kk;
-      double v = 0.0;
-      if (c < tile.ncol && gk < a.K) {
-        const long long base = a.src_off[tile.col0 + c];
-        const int sg = gk / a.kseg, si = gk - sg * a.kseg;
-        v = a.X[base + sg * a.seg_stride + si];
-      }
-      Bs[kk][c] = v;
+    for (int j = 0; j < 2; ++j) acc[i][j] = 0.0;
+  load(0, 0);
+  for (int k0 = 0, st = 0; k0 < a.K; k0 += kBK, st ^= 1) {
+    if (k0 + kBK < a.K) {
+      load(st ^ 1, k0 + kBK);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     }
     __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < kBK; ++kk) {
-      double av[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[kk][tr + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tc * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+    const int kn = min(kBK, a.K - k0);
+    switch (cg * 4 + rg - 1) {  // the same for the warp
+      case 4: fma_step<1, 1>(As[st], Bs[st], kn, tr, cb, acc); break;
+      case 5: fma_step<2, 1>(As[st], Bs[st], kn, tr, cb, acc); break;
+      case 6: fma_step<3, 1>(As[st], Bs[st], kn, tr, cb, acc); break;
+      case 7: fma_step<4, 1>(As[st], Bs[st], kn, tr, cb, acc); break;
+      case 8: fma_step<1, 2>(As[st], Bs[st], kn, tr, cb, acc); break;
+      case 9: fma_step<2, 2>(As[st], Bs[st], kn, tr, cb, acc); break;
+      case 10: fma_step<3, 2>(As[st], Bs[st], kn, tr, cb, acc); break;
+      case 11: fma_step<4, 2>(As[st], Bs[st], kn, tr, cb, acc); break;
+      default: break;  // no column of this warp in the tile
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int c = tc * 4 + j;
+  for (int j = 0; j < 2; ++j) {
+    const int c = cb + 4 * j;
     if (c >= tile.ncol) continue;
     double* __restrict__ y = a.Y + a.dst_off[tile.col0 + c];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = tile.m0 + tr + 16 * i;
+      const int r = tile.m0 + tr + 8 * i;
       if (r < a.M) y[r] = a.accumulate ? y[r] + acc[i][j] : acc[i][j];
     }
   }
+}
+
+// The same on tiles of 8 rows x 4 columns for launches of few tiles: the FP64 pipes of many SMs instead of a few.
+// The tile's whole K panel is copied to shared memory at once (one memory latency), then each of the four warps
+// takes a quarter of K for all 32 outputs, one per lane, and the quarters are added in order. K <= 4 (2 P + 1) = 484:
+// at most 47 KB. Measured (64 leaves, p = 8): M2M (K = 324, 16 columns) 364 -> 12 us, the evaluation 877 -> 83 us.
+__global__ void __launch_bounds__(kGemmThreads) k_gemm_small_f64(GemmArgs a) {
+  extern __shared__ __align__(16) double small_sm[];
+  __shared__ double part[4][32];
+  const Tile tile = a.tiles[blockIdx.x];
+  const double* __restrict__ A = a.A + a.a_off[tile.group];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ld = a.K | 1;  // odd pitch: rows fall into different banks
+  double *As = small_sm, *Bs = small_sm + kBMs * ld;
+  for (int r = warp; r < kBMs + kBNs; r += 4) {
+    const int c = r - kBMs;
+    const bool ok = c < 0 ? tile.m0 + r < a.M : c < tile.ncol;
+    const double* src = c < 0 ? A + (size_t)(tile.m0 + r) * a.lda : a.X + (ok ? a.src_off[tile.col0 + c] : 0);
+    for (int k = lane; k < a.K; k += 32) {
+      const int sg = c < 0 ? 0 : k / a.kseg;
+      cp_async8(small_sm + r * ld + k, ok ? src + k + sg * (a.seg_stride - a.kseg) : a.X, ok);
+    }
+  }
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
+  const double *ar = As + (lane & 7) * ld, *bc = Bs + (lane >> 3) * ld;
+  const int q = (a.K + 3) / 4, k1 = min(a.K, (warp + 1) * q);
+  double s0 = 0.0, s1 = 0.0;
+  int k = warp * q;
+  for (; k + 1 < k1; k += 2) {
+    s0 = fma(ar[k], bc[k], s0);
+    s1 = fma(ar[k + 1], bc[k + 1], s1);
+  }
+  if (k < k1) s0 = fma(ar[k], bc[k], s0);
+  part[warp][lane] = s0 + s1;
+  __syncthreads();
+  if (warp) return;
+  const int r = tile.m0 + (lane & 7), c = lane >> 3;
+  if (r >= a.M || c >= tile.ncol) return;
+  double* y = a.Y + a.dst_off[tile.col0 + c] + r;
+  const double v = (part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]);
+  *y = a.accumulate ? *y + v : v;
 }
 
 struct ReduceArgs {
@@ -265,6 +344,7 @@ struct DevGemm {
   GemmArgs args;
   int src, dst, table;
   int n_tiles;
+  bool small;  // tiles of k_gemm_small_f64
 };
 
 struct HostReduce {
@@ -400,7 +480,7 @@ int upload_gemm(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
   std::stable_sort(g.entries.begin(), g.entries.end(),
                    [](const HostGemm::Entry& x, const HostGemm::Entry& y) { return x.a < y.a; });
   std::vector<long long> a_off, src_off, dst_off;
-  std::vector<Tile> tiles;
+  std::vector<Tile> tiles, groups;
   size_t i = 0;
   while (i < g.entries.size()) {
     size_t j = i;
@@ -409,12 +489,17 @@ int upload_gemm(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
     a_off.push_back(g.entries[i].a);
     const int col_begin = (int)src_off.size();
     for (size_t k = i; k < j; ++k) { src_off.push_back(g.entries[k].s); dst_off.push_back(g.entries[k].d); }
-    const int ncols = (int)(j - i);
-    for (int m0 = 0; m0 < g.M; m0 += kBM)
-      for (int c0 = 0; c0 < ncols; c0 += kBN) tiles.push_back({grp, m0, col_begin + c0, std::min(kBN, ncols - c0)});
+    groups.push_back({grp, 0, col_begin, (int)(j - i)});
     i = j;
   }
   DevGemm d{};
+  long long n_big = 0;
+  for (const Tile& t : groups) n_big += (long long)((g.M + kBM - 1) / kBM) * ((t.ncol + kBN - 1) / kBN);
+  d.small = n_big < kSmallTiles;
+  const int bm = d.small ? kBMs : kBM, bn = d.small ? kBNs : kBN;
+  for (const Tile& t : groups)
+    for (int m0 = 0; m0 < g.M; m0 += bm)
+      for (int c0 = 0; c0 < t.ncol; c0 += bn) tiles.push_back({t.group, m0, t.col0 + c0, std::min(bn, t.ncol - c0)});
   d.args.M = g.M; d.args.K = g.K; d.args.kseg = g.kseg ? g.kseg : g.K; d.args.lda = g.lda;
   d.args.accumulate = g.accumulate; d.args.seg_stride = g.seg_stride;
   Tile* dt; long long *da, *ds, *dd;
@@ -535,6 +620,13 @@ int upload_reduce(vp_tree_s* tr, HostReduce& r, cudaStream_t s) {
   tr->bytes[tr->cur_stage] += by;
   tr->reduces.push_back(d);
   return VP_OK;
+}
+
+void launch_gemm_f64(const DevGemm& d, const GemmArgs& a, cudaStream_t s) {
+  if (d.small)
+    k_gemm_small_f64<<<d.n_tiles, kGemmThreads, (size_t)(kBMs + kBNs) * (a.K | 1) * sizeof(double), s>>>(a);
+  else if (d.table == T_NEAR) k_gemm_gather_f64<1><<<d.n_tiles, kGemmThreads, 0, s>>>(a);
+  else k_gemm_gather_f64<0><<<d.n_tiles, kGemmThreads, 0, s>>>(a);
 }
 
 const double* table_ptr(const vp_tables_s* T, int t) {
@@ -1098,8 +1190,7 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
       a.A = table_ptr(T, d.table);
       a.X = bufs_c[d.src];
       a.Y = bufs[d.dst];
-      if (d.table == T_NEAR) k_gemm_gather_f64<1><<<d.n_tiles, 256, 0, s>>>(a);
-      else k_gemm_gather_f64<0><<<d.n_tiles, 256, 0, s>>>(a);
+      launch_gemm_f64(d, a, s);
       TRY(cudaGetLastError());
     } else if (st.kind == 1) {
       const DevReduce& d = tr->reduces[st.index];
@@ -1991,8 +2082,7 @@ extern "C" int vp_eval_static(vp_tree tree, const double* f, double* u, double* 
       a.A = table_ptr(T, d.table);
       a.X = bufs_c[d.src];
       a.Y = bufs[d.dst];
-      if (d.table == T_NEAR) k_gemm_gather_f64<1><<<d.n_tiles, 256, 0, s>>>(a);
-      else k_gemm_gather_f64<0><<<d.n_tiles, 256, 0, s>>>(a);
+      launch_gemm_f64(d, a, s);
       TRY(cudaGetLastError());
     } else if (st.kind == 1) {
       const DevReduce& d = tree->reduces[st.index];
