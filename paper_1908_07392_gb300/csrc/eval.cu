@@ -522,6 +522,16 @@ int upload_gemm(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
   return VP_OK;
 }
 
+// Engine of a launch that vp_autotune has not timed (layer potentials, and trees that are not tuned): the tensor-memory
+// engines, on 128 x 128 tiles (transposed for operators of at most 128 rows) where that gives every SM two tiles, on
+// 128 x 64 tiles below. The autotuner's choices on the full-size star and the coupled-step layer follow this
+// line but for a few launches within 10 %; mma.sync, the choice before, takes 2.1 to 3.3 times as long on the layer's
+// large launches (M2L 274 -> 94 us, L2T 281 -> 84, last L2L 213 -> 127) and 1.1 to 1.6 times on its small ones.
+int default_engine(int M, int tiles128) {
+  if (tiles128 < 304) return kEngineTcgen05N64;
+  return M <= 128 ? kEngineTcgen05T : kEngineTcgen05;
+}
+
 // Split-precision contraction: the same grouping, with tiles of the tensor-core kernel, matrix indices
 // instead of element offsets and vector indices instead of source offsets.
 int upload_split(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
@@ -567,6 +577,7 @@ int upload_split(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
   if ((rc = dev_upload(tr, dst_off, &dd, s))) return rc;
   d.args.a_mat = da; d.args.src_vec = ds; d.args.dst_off = dd;
   d.table = g.table; d.vec = g.split_vec; d.dst = g.dst;
+  d.engine = default_engine(g.M, d.n_tiles[kEngineTcgen05]);
   // algorithmic bytes: sliced operators (S bf16 slices + a row exponent) and sliced source vectors
   // (S slices + an exponent) read once, outputs written once (8 bytes: a double-float slot or FP64)
   const int kp = split_kpad(g.K);
@@ -649,6 +660,9 @@ const double* table_ptr(const vp_tables_s* T, int t) {
 int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   const vp_tables_s* T = tr->T;
   const int n = T->n, C = T->C, E = T->E, nch = T->nch;
+  const bool split = T->precision == VP_PREC_SPLIT;
+  // slot strides: even in split precision, whose reduction reads two rows at a time
+  const int Cs = split ? (C + 1) & ~1 : C, Us = split ? (3 * n + 1) & ~1 : 3 * n;
   const auto& B = P.boxes;
   const long long NB = (long long)B.size();
   auto kact = [&](int l) { return l >= 0 && l <= T->levels && T->kactive[l]; };
@@ -664,9 +678,9 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
     for (int ch = 0; ch < nch; ++ch) {
       if (ch == 0 && !kact(l)) continue;
       const long long slot = nls++;
-      lsl[(size_t)v.tgt * nch + ch].push_back(slot * C);
+      lsl[(size_t)v.tgt * nch + ch].push_back(slot * Cs);
       m2l.entries.push_back({(long long)(l * T->m2l_stride_lvl() + v.pos * T->m2l_stride_off() + ch * T->m2l_stride_ch()),
-                             (long long)v.src * E + ch * C, slot * C});
+                             (long long)v.src * E + ch * C, slot * Cs});
     }
   }
   s2l.M = C; s2l.K = n; s2l.lda = n; s2l.table = T_S2L; s2l.src = BUF_F; s2l.dst = BUF_LSLOT; s2l.split_vec = 0;
@@ -675,9 +689,9 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
     for (int ch = 0; ch < nch; ++ch) {
       if (ch == 0 && !kact(l)) continue;
       const long long slot = nls++;
-      lsl[(size_t)x.tgt * nch + ch].push_back(slot * C);
+      lsl[(size_t)x.tgt * nch + ch].push_back(slot * Cs);
       s2l.entries.push_back({(long long)(l * T->s2l_stride_lvl() + x.pos * T->s2l_stride_pos() + ch * T->s2l_stride_ch()),
-                             (long long)B[x.src].leaf * n, slot * C});
+                             (long long)B[x.src].leaf * n, slot * Cs});
     }
   }
   nearg.M = 3 * n; nearg.K = n; nearg.lda = n; nearg.table = T_NEAR; nearg.src = BUF_F; nearg.dst = BUF_USLOT;
@@ -685,9 +699,9 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   for (const Pair& u : P.U) {
     const int l = B[u.tgt].level;
     const long long slot = nus++;
-    usl[u.tgt].push_back(slot * 3 * n);
+    usl[u.tgt].push_back(slot * Us);
     nearg.entries.push_back({(long long)(l * T->near_stride_lvl() + u.pos * T->near_stride_pos()),
-                             (long long)B[u.src].leaf * n, slot * 3 * n});
+                             (long long)B[u.src].leaf * n, slot * Us});
   }
   m2t.M = 3 * n; m2t.K = C; m2t.lda = C; m2t.table = T_M2T; m2t.src = BUF_MP; m2t.dst = BUF_USLOT; m2t.split_vec = 1;
   for (const Pair& w : P.W) {
@@ -695,9 +709,9 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
     for (int ch = 0; ch < nch; ++ch) {
       if (ch == 0 && !kact(l + 1)) continue;
       const long long slot = nus++;
-      usl[w.tgt].push_back(slot * 3 * n);
+      usl[w.tgt].push_back(slot * Us);
       m2t.entries.push_back({(long long)(l * T->m2t_stride_lvl() + w.pos * T->m2t_stride_pos() + ch * T->m2t_stride_ch()),
-                             (long long)w.src * E + ch * C, slot * 3 * n});
+                             (long long)w.src * E + ch * C, slot * Us});
     }
   }
   l2t.M = 3 * n; l2t.K = E; l2t.lda = E; l2t.table = T_L2T; l2t.src = BUF_LOC; l2t.dst = BUF_USLOT; l2t.split_vec = 2;
@@ -707,8 +721,8 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
     const Box& b = B[i];
     if (b.leaf < 0 || b.level < 2) continue;
     const long long slot = nus++;
-    usl[i].push_back(slot * 3 * n);
-    l2t.entries.push_back({(long long)(b.level * T->l2t_stride_lvl()), i * E, slot * 3 * n});
+    usl[i].push_back(slot * Us);
+    l2t.entries.push_back({(long long)(b.level * T->l2t_stride_lvl()), i * E, slot * Us});
     s2m.entries.push_back({(long long)(b.level * T->s2m_stride_lvl()), (long long)b.leaf * n, i * E});
   }
   tr->n_lslot = nls;
@@ -719,11 +733,10 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   tr->allocs.push_back(tr->mp);
   TRY(cudaMalloc(&tr->loc, std::max<long long>(1, NB * E) * sizeof(double)));
   tr->allocs.push_back(tr->loc);
-  TRY(cudaMalloc(&tr->lslot, std::max<long long>(1, nls * C) * sizeof(double)));
+  TRY(cudaMalloc(&tr->lslot, std::max<long long>(1, nls * Cs) * sizeof(double)));
   tr->allocs.push_back(tr->lslot);
-  TRY(cudaMalloc(&tr->uslot, std::max<long long>(1, nus * 3 * n) * sizeof(double)));
+  TRY(cudaMalloc(&tr->uslot, std::max<long long>(1, nus * Us) * sizeof(double)));
   tr->allocs.push_back(tr->uslot);
-  const bool split = T->precision == VP_PREC_SPLIT;
   if (split) {
     // sliced source vectors of every family
     const long long nv[kVecFamilies] = {tr->n_leaves, NB * nch, NB, NB * nch, NB * nch, NB * nch};

@@ -103,33 +103,71 @@ __global__ void k_slice_rows(const double* __restrict__ A, long long mstride, in
 }
 
 // Slice a list of vectors. Vector v (v < nlist) has identifier id = vid ? vid[v] : v and elements
-// x_k = X[b + (k / kseg) * seg_stride + k % kseg], k < K, b = base ? base[v] : v * cstride;
+// x_k = X[b + (k / kseg) * seg_stride + k % kseg], k < K <= 2 kseg, b = base ? base[v] : v * cstride;
 // output out[id][Kpad / 16][s][16] (the S slices of each K step of 16 are contiguous, so one
-// column of a K step is one 32 S-byte block for the GEMM engines' gathers) and eb[id]. One warp
-// per vector.
+// column of a K step is one 32 S-byte block for the GEMM engines' gathers) and eb[id].
+//
+// L lanes per vector (a power of two, L >= Kpad / 8), a lane taking 8 consecutive elements: they are read once and
+// kept for the digits, and a slice of them is one 16-byte store (2-byte stores, six per element, and a second
+// read of the vector took 571 us an evaluation of the full-size star, now 459). The digits are those of digits(): with 128 added to each of the lower five,
+// balanced digits are plain bytes, and a byte under the bits of 2^23 is a float that one multiply-add turns into
+// (byte - 128) 2^(-8 (i + 1)), exact. Measured: the star's leaf sources (40,897 vectors of 256) 79 -> 52 us = 4.0 TB/s.
 template <int S>
-__global__ void k_slice_list(const double* __restrict__ X, const long long* __restrict__ base,
-                             const long long* __restrict__ vid, long long nlist, int K, int kseg,
-                             long long seg_stride, long long cstride, int Kpad, slice_t* __restrict__ out,
-                             int* __restrict__ eb) {
-  const long long v = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (v >= nlist) return;
-  const long long b = base ? base[v] : v * cstride;
-  const long long id = vid ? vid[v] : v;
+__global__ void __launch_bounds__(256) k_slice_list(const double* __restrict__ X, const long long* __restrict__ base,
+                                                    const long long* __restrict__ vid, long long nlist, int K, int kseg,
+                                                    long long seg_stride, long long cstride, int Kpad, int lg_l,
+                                                    slice_t* __restrict__ out, int* __restrict__ eb) {
+  static_assert(S == 6, "five balanced bytes and a leading digit");
+  const int L = 1 << lg_l, l = threadIdx.x & (L - 1);
+  const long long v = (blockIdx.x * 256ll + threadIdx.x) >> lg_l;
+  const bool ok = v < nlist;
+  const long long b = !ok ? 0 : (base ? base[v] : v * cstride);
+  double x[8];
   double mx = 0.0;
-  for (int k = lane; k < K; k += 32) {
-    const int sg = k / kseg;
-    mx = fmax(mx, fabs(X[b + sg * seg_stride + (k - sg * kseg)]));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = 8 * l + i;
+    x[i] = ok && k < K ? X[b + k + (k >= kseg ? seg_stride - kseg : 0)] : 0.0;
+    mx = fmax(mx, fabs(x[i]));
   }
-  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  for (int o = L >> 1; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (!ok || 8 * l >= Kpad) return;
   const int e = exponent_of(mx);
-  slice_t* o = out + id * (long long)S * Kpad;
-  for (int k = lane; k < Kpad; k += 32) {
-    const int sg = k / kseg;
-    digits<S>(k < K ? X[b + sg * seg_stride + (k - sg * kseg)] : 0.0, e, o + (k >> 4) * (S * 16) + (k & 15), 16);
+  const long long id = vid ? vid[v] : v;
+  if (l == 0) eb[id] = e;
+  unsigned w[S][4];
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {
+    unsigned long long T[2];
+    unsigned sign = 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const unsigned long long bits = (unsigned long long)__double_as_longlong(x[i + q]);
+      int ex = (int)((bits >> 52) & 0x7ff);
+      unsigned long long m = bits & ((1ull << 52) - 1);
+      if (ex) m |= 1ull << 52;
+      else ex = 1;
+      const int sh = ex - 1075 + 8 * S - e;
+      if (m == 0 || sh <= -64) T[q] = 0;
+      else if (sh >= 0) T[q] = m << sh;
+      else T[q] = (m + (1ull << (-sh - 1))) >> (-sh);
+      T[q] += 0x8080808080ull;
+      sign |= (unsigned)(bits >> 63) << (15 + 16 * q);
+    }
+#pragma unroll
+    for (int d = 0; d < S; ++d) {
+      const int at = 8 * (S - 1 - d);  // bit position of digit d
+      const unsigned keep = d == 0 ? 0xffffu : 0xffu;
+      const float f0 = __uint_as_float(0x4b000000u | ((unsigned)(T[0] >> at) & keep));
+      const float f1 = __uint_as_float(0x4b000000u | ((unsigned)(T[1] >> at) & keep));
+      const float sc = __int_as_float((127 - 8 * (d + 1)) << 23), off = -(8388608.f + (d == 0 ? 0.f : 128.f)) * sc;
+      const __nv_bfloat162 p = __floats2bfloat162_rn(fmaf(f0, sc, off), fmaf(f1, sc, off));
+      w[d][i >> 1] = *reinterpret_cast<const unsigned*>(&p) ^ sign;
+    }
   }
-  if (lane == 0) eb[id] = e;
+  slice_t* o = out + id * (long long)S * Kpad + (l >> 1) * (S * 16) + (l & 1) * 8;
+#pragma unroll
+  for (int d = 0; d < S; ++d) *reinterpret_cast<uint4*>(o + d * 16) = make_uint4(w[d][0], w[d][1], w[d][2], w[d][3]);
 }
 
 __device__ inline void df_add(float& hi, float& lo, float x) {
@@ -924,55 +962,58 @@ size_t tc_smem_bytes(int S, int BN) { return (size_t)kTcStages * S * (kTcA + BN 
 
 // ------------------------------------------------------------------ reduction
 
-// Reduction of double-float slots: y[dst] = sum of slots (double-float), written as FP64.
-__global__ void k_reduce_df(DFReduceArgs a) {
-  constexpr int kChunk = 64;  // slot offsets staged in shared memory per pass
-  __shared__ long long slot_sh[kChunk];
-  const int d = blockIdx.x;
+// Reduction of double-float slots: y[dst] = sum of its slots (double-float, in slot order), written as FP64. A thread
+// sums two neighbouring rows (16-byte reads: slots start at even offsets), `per` threads a destination, as many
+// destinations to a block as fit; slot offsets come through L1 by broadcast, so a block waits for no barrier (one
+// destination per block of 256 threads, offsets staged in shared memory, left short destinations waiting on
+// latency: the coupled-step layer's output, 1 to 2 slots of 256 rows, 133 -> 51 us; long ones stream slots at the copy
+// rate either way, the full-size star's output 559 -> 580 us. More loads in flight cost occupancy: 6 took 782 us).
+template <bool FINAL>
+__global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, int per, int vec_out) {
+  const int sub = threadIdx.x / per, t = threadIdx.x - sub * per;
+  const int d = blockIdx.x * (blockDim.x / per) + sub, r = 2 * t;
+  if (d >= n_dst || r >= a.M) return;
   const long long b = a.ptr[d], e = a.ptr[d + 1];
-  const float2* S = reinterpret_cast<const float2*>(a.S);
-  const int rows_per_pass = (a.M + blockDim.x - 1) / blockDim.x;
-  // each thread owns up to 4 rows (M <= 4 * blockDim.x), summed in slot order
-  float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-  for (long long c0 = b; c0 < e; c0 += kChunk) {
-    const int nc = (int)((e - c0) < kChunk ? (e - c0) : kChunk);
-    __syncthreads();
-    if (threadIdx.x < nc) slot_sh[threadIdx.x] = a.slot[c0 + threadIdx.x];
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (q >= rows_per_pass) break;
-      const int r = threadIdx.x + q * blockDim.x;
-      if (r >= a.M) break;
-      int k = 0;
-      for (; k + 4 <= nc; k += 4) {  // four loads in flight, added in slot order
-        const float2 v0 = S[slot_sh[k] + r], v1 = S[slot_sh[k + 1] + r];
-        const float2 v2 = S[slot_sh[k + 2] + r], v3 = S[slot_sh[k + 3] + r];
-        df_add(hi[q], lo[q], v0.x); df_add(hi[q], lo[q], v0.y);
-        df_add(hi[q], lo[q], v1.x); df_add(hi[q], lo[q], v1.y);
-        df_add(hi[q], lo[q], v2.x); df_add(hi[q], lo[q], v2.y);
-        df_add(hi[q], lo[q], v3.x); df_add(hi[q], lo[q], v3.y);
-      }
-      for (; k < nc; ++k) {
-        const float2 v = S[slot_sh[k] + r];
-        df_add(hi[q], lo[q], v.x);
-        df_add(hi[q], lo[q], v.y);
-      }
-    }
+  const float2* S = reinterpret_cast<const float2*>(a.S) + r;
+  float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+  auto add = [&](float4 v) {
+    df_add(h0, l0, v.x); df_add(h0, l0, v.y);
+    df_add(h1, l1, v.z); df_add(h1, l1, v.w);
+  };
+  auto at = [&](long long o) { return __ldcs(reinterpret_cast<const float4*>(S + o)); };
+  long long k = b;
+  for (; k + 4 <= e; k += 4) {  // four loads in flight, added in slot order
+    const long long o0 = __ldg(a.slot + k), o1 = __ldg(a.slot + k + 1), o2 = __ldg(a.slot + k + 2), o3 = __ldg(a.slot + k + 3);
+    const float4 v0 = at(o0), v1 = at(o1), v2 = at(o2), v3 = at(o3);
+    add(v0); add(v1); add(v2); add(v3);
   }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = threadIdx.x + q * blockDim.x;
-    if (q >= rows_per_pass || r >= a.M) break;
-    const double s = (double)hi[q] + (double)lo[q];
-    if (a.final_out) {
-      const int f = r / a.n, t = r - f * a.n;
-      const long long o = a.dst_off[d] + t;
-      if (f == 0) a.u[o] = s;
-      else a.g[(f - 1) * a.N + o] = s;
-    } else {
-      a.Y[a.dst_off[d] + r] = s;
+  if (k < e) {
+    const long long n1 = k + 1 < e ? k + 1 : k, n2 = k + 2 < e ? k + 2 : k;
+    const long long o0 = __ldg(a.slot + k), o1 = __ldg(a.slot + n1), o2 = __ldg(a.slot + n2);
+    const float4 v0 = at(o0), v1 = at(o1), v2 = at(o2);
+    add(v0);
+    if (k + 1 < e) add(v1);
+    if (k + 2 < e) add(v2);
+  }
+  const double y0 = (double)h0 + (double)l0, y1 = (double)h1 + (double)l1;
+  double* y;
+  if (FINAL) {
+    const int f = r / a.n;
+    y = (f == 0 ? a.u : a.g + (f - 1) * a.N) + a.dst_off[d] + (r - f * a.n);
+    if (!vec_out && r + 1 < a.M) {  // the next row may begin another field
+      const int f1 = (r + 1) / a.n;
+      (f1 == 0 ? a.u : a.g + (f1 - 1) * a.N)[a.dst_off[d] + (r + 1 - f1 * a.n)] = y1;
+      *y = y0;
+      return;
     }
+  } else {
+    y = a.Y + a.dst_off[d] + r;
+  }
+  if (vec_out) {
+    *reinterpret_cast<double2*>(y) = make_double2(y0, y1);
+  } else {
+    y[0] = y0;
+    if (!FINAL && r + 1 < a.M) y[1] = y1;
   }
 }
 
@@ -1109,17 +1150,29 @@ int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engin
 int launch_slice_list(const double* X, const long long* base, const long long* vid, long long nlist, int K, int kseg,
                       long long seg_stride, long long cstride, void* out, int* eb, cudaStream_t s) {
   if (nlist <= 0) return VP_OK;
-  k_slice_list<kSplitSlices><<<(unsigned)((nlist * 32 + 255) / 256), 256, 0, s>>>(
-      X, base, vid, nlist, K, kseg > 0 ? kseg : K, seg_stride, cstride, kpad(K), (slice_t*)out, eb);
+  int lg_l = 2;  // lanes per vector: at least Kpad / 8, which is at most 32
+  while ((8 << lg_l) < kpad(K)) ++lg_l;
+  if (lg_l > 5 || (kseg > 0 && K > 2 * kseg)) return VP_ERR_ARG;
+  k_slice_list<kSplitSlices><<<(unsigned)(((nlist << lg_l) + 255) / 256), 256, 0, s>>>(
+      X, base, vid, nlist, K, kseg > 0 ? kseg : K, seg_stride, cstride, kpad(K), lg_l, (slice_t*)out, eb);
   TRY(cudaGetLastError());
   return VP_OK;
 }
 
 int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s) {
   if (n_dst <= 0) return VP_OK;
-  const int threads = a.M >= 256 ? 256 : ((a.M + 31) / 32) * 32;
-  if (a.M > 4 * threads) return VP_ERR_ARG;  // rows per thread are held in registers (3 p^2 <= 768)
-  k_reduce_df<<<n_dst, threads, 0, s>>>(a);
+  const int pairs = (a.M + 1) / 2;
+  if (pairs > 512) return VP_ERR_ARG;  // 3 p^2 <= 768 rows
+  // threads of a destination: whole warps from 32 on, so that a destination's reads stay coalesced
+  const int per = (pairs + 31) / 32 * 32, threads = per >= 96 ? per : 128 / per * per;
+  const unsigned blocks = (unsigned)((n_dst + threads / per - 1) / (threads / per));
+  auto even = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  if (a.final_out) {
+    // n even: a pair of rows lies in one field, and destinations and N are even too
+    k_reduce_df<true><<<blocks, threads, 0, s>>>(a, n_dst, per, a.n % 2 == 0 && even(a.u) && even(a.g));
+  } else {
+    k_reduce_df<false><<<blocks, threads, 0, s>>>(a, n_dst, per, 0);
+  }
   TRY(cudaGetLastError());
   return VP_OK;
 }
