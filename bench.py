@@ -425,7 +425,7 @@ def layer_and_periodic(args, V):
         flush.zero_(); torch.cuda.synchronize()
         launches = V.vp_layer_steps(layer, mu, u)
         kinds = {0: "fp64 gemm", 1: "fp64 reduce", 2: "memset", 3: "slice", 4: "split gemm", 5: "df reduce",
-                 6: "point operator"}
+                 6: "point operator", 7: "near correction", 8: "sum and slice"}
         top = sorted(launches, key=lambda x: -x["ms"])[:6]
         med = statistics.median(ms)
         out["layer_potential"] = {
@@ -752,9 +752,8 @@ def measure(args, V, w, prec, world, local, with_e2e):
             ms_k = statistics.mean(m[k] for m in stage_ms)
             stage_roof[name] = dict(rate(stage_flops[k], stage_bytes[k], ms_k), gflop=round(stage_flops[k] / 1e9, 2),
                                     gbytes=round(stage_bytes[k] / 1e9, 3))
-        kinds = {0: "fp64 gemm", 1: "fp64 reduce", 2: "memset", 3: "slice", 4: "split gemm", 5: "df reduce"}
-        tables = {-1: "-", 0: "near", 1: "s2m", 2: "l2t", 3: "m2m", 4: "l2l", 5: "m2l", 6: "m2t", 7: "s2l",
-                  8: "m2m_lo", 9: "m2m_hi"}
+        kinds = {0: "fp64 gemm", 1: "fp64 reduce", 2: "memset", 3: "slice", 4: "split gemm", 5: "df reduce", 8: "sum and slice"}
+        tables = {-1: "-", 0: "near", 1: "s2m", 2: "l2t", 3: "m2m", 4: "l2l", 5: "m2l", 6: "m2t", 7: "s2l"}
         top = sorted(range(len(launch_list)), key=lambda i: -launch_list[i]["ms"])[:10]
         top_launches = [dict(rate(launch_list[i]["flops"], launch_list[i]["bytes"], launch_list[i]["ms"]),
                              index=i, kind=kinds.get(launch_list[i]["kind"], "?"),

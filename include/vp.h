@@ -210,7 +210,7 @@ int vp_eval_timed(vp_tree tree, const double* f, double* u, double* gradu, void*
 
 /*
  * vp_tree_stats -- static work of one evaluation of `tree`:
- *  launches     number of kernel launches (and memsets) one vp_eval issues;
+ *  launches     number of kernel launches (and, for FP64, a memset) one vp_eval issues;
  *  stage_flops  host array [VP_NSTAGES]: algorithmic floating-point operations
  *               per stage (2*M*K per column of each contraction, one add per
  *               reduced element). Either pointer may be NULL.
@@ -232,7 +232,7 @@ int vp_tree_bytes(vp_tree tree, double* stage_bytes);
  * *n_steps (the number of launches, including memsets) is returned. Otherwise cap >= *n_steps and
  * the host arrays receive, per launch k: ms[k] (milliseconds), info[4k..4k+3] = (kind: 0 FP64
  * contraction, 1 FP64 reduction, 2 memset, 3 slicing, 4 split contraction, 5 double-float
- * reduction; stage VP_STAGE_*; operator table id or -1; split engine or -1), flops[k] and
+ * reduction, 6 point-source operator, 7 near-boundary correction, 8 slots summed and sliced; stage VP_STAGE_*; operator table id or -1; split engine or -1), flops[k] and
  * bytes[k] (algorithmic, as vp_tree_stats and vp_tree_bytes count them). Same device arguments
  * as vp_eval. Errors: VP_ERR_ARG, VP_ERR_CUDA.
  */

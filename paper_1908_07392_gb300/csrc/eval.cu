@@ -14,6 +14,9 @@
 //   S2L (X lists) into local slots -> reduce into local expansions ->
 //   L2L (coarsest first) -> L2T, M2T (W lists) and near tables (U lists) into
 //   output slots -> reduce into u, du/dx, du/dy.
+// In split precision every contraction writes slots, M2M and L2L too, and the
+// expansions of a level are summed from them and sliced by one launch
+// (k_sum_slice): they exist only as slots and digits.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -332,9 +335,7 @@ struct HostGemm {
   long long seg_stride = 0;
   int table = 0;  // which table array
   int src = 0, dst = 0;
-  // split precision: source vector family (-1: always FP64; 0: leaf values, 1: (box, channel)
-  // multipoles, 2: box locals) and output (0: double-float slot, 1: FP64 overwrite, 2: FP64 accumulate)
-  int split_vec = -1, out_mode = 0;
+  int split_vec = -1;       // split precision: source vector family (kVecFamilies)
   long long mat_elems = 0;  // elements of one operator matrix (0: M * lda; set when M is a leading part)
   struct Entry { long long a, s, d, v = -1; };  // v: sliced-vector id (split), -1 = derived from s
   std::vector<Entry> entries;
@@ -366,9 +367,8 @@ struct DevSplit {
 };
 
 // Sliced-vector families (split precision): 0 leaf values (K = n), 1 (box, channel) multipoles (K = C),
-// 2 box locals (K = E), 3 multipoles of children 0-1 of (parent, channel) (K = 2C), 4 (box, channel)
-// locals (K = C), 5 multipoles of children 2-3 of (parent, channel) (K = 2C).
-constexpr int kVecFamilies = 6;
+// 2 locals of leaves (K = E), 3 (box, channel) locals of internal boxes (K = C).
+constexpr int kVecFamilies = 4;
 struct DevSlice {
   int family, buf, K, kseg;
   long long seg_stride, cstride, n;
@@ -376,7 +376,22 @@ struct DevSlice {
   const long long* vid;   // null: identity
 };
 
-enum Table { T_NEAR, T_S2M, T_L2T, T_M2M, T_L2L, T_M2L, T_M2T, T_S2L, T_M2M_LO, T_M2M_HI };
+enum Table { T_NEAR, T_S2M, T_L2T, T_M2M, T_L2L, T_M2L, T_M2T, T_S2L };
+
+// Sums of contribution slots (buffer `buf`) sliced into a family: n vectors of nseg segments of C elements.
+struct DevSum {
+  int family, buf, nseg;
+  long long n;
+  const long long *ptr, *slot, *vid;
+};
+struct HostSum {
+  int family = 0, buf = 0, nseg = 1;
+  std::vector<long long> ptr{0}, slot, vid;
+  void segment(const std::vector<long long>& slots) {
+    slot.insert(slot.end(), slots.begin(), slots.end());
+    ptr.push_back((long long)slot.size());
+  }
+};
 
 // A point-source operator launch (layer potential): instances of small dense matrices applied to the
 // boundary density (layer.h), written into buffer `dst`.
@@ -398,7 +413,7 @@ struct DevNear {
 
 struct Step {
   int kind;   // 0 gemm, 1 reduce, 2 memset mp, 3 slice vectors, 4 split gemm, 5 double-float reduce,
-              // 6 point-source operator, 7 near-boundary correction of the output
+              // 6 point-source operator, 7 near-boundary correction of the output, 8 slots summed and sliced
   int index;
   int stage;  // VP_STAGE_* for timing
   double flops = 0.0;  // algorithmic floating-point operations of the step
@@ -430,6 +445,8 @@ struct vp_tree_s {
   void* sv[vp::kVecFamilies] = {nullptr};
   int* se[vp::kVecFamilies] = {nullptr};
   std::vector<vp::DevSlice> slice_ops;
+  std::vector<vp::DevSum> sums;
+  bool pdl = false;         // the chain's launches overlap (programmatic dependent launch)
   // host staging for vp_eval_host
   double *h_f = nullptr, *h_u = nullptr;
   double *d_f = nullptr, *d_u = nullptr, *d_g = nullptr;
@@ -563,7 +580,7 @@ int upload_split(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
     i = j;
   }
   DevSplit d{};
-  d.args.M = g.M; d.args.Kpad = split_kpad(g.K); d.args.out_mode = g.out_mode;
+  d.args.M = g.M; d.args.Kpad = split_kpad(g.K);
   long long *da, *ds, *dd;
   int rc;
   for (int en = 0; en < kEngines; ++en) {
@@ -584,7 +601,7 @@ int upload_split(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
   const double fl = 2.0 * g.M * (double)g.K * (double)g.entries.size();
   const double by = (double)a_mat.size() * g.M * (2.0 * kSplitSlices * kp + 4.0) +
                     (double)count_distinct(src_vec) * (2.0 * kSplitSlices * kp + 4.0) +
-                    8.0 * (1.0 + (g.out_mode == 2)) * (double)g.entries.size() * g.M;
+                    8.0 * (double)g.entries.size() * g.M;
   tr->steps.push_back({4, (int)tr->splits.size(), tr->cur_stage, fl, by});
   tr->splits.push_back(d);
   tr->flops[tr->cur_stage] += fl;
@@ -605,6 +622,28 @@ int add_slice(vp_tree_s* tr, int family, int buf, int K, int kseg, long long seg
   tr->steps.push_back({3, (int)tr->slice_ops.size(), tr->cur_stage, 0.0, by});
   tr->bytes[tr->cur_stage] += by;
   tr->slice_ops.push_back(d);
+  return VP_OK;
+}
+
+// A sum-and-slice step.
+int upload_sum(vp_tree_s* tr, const HostSum& h, cudaStream_t s) {
+  if (h.vid.empty()) return VP_OK;
+  const int C = tr->T->C;
+  DevSum d{h.family, h.buf, h.nseg, (long long)h.vid.size(), nullptr, nullptr, nullptr};
+  long long* p = nullptr;
+  int rc;
+  if ((rc = dev_upload(tr, h.ptr, &p, s))) return rc;
+  d.ptr = p;
+  if ((rc = dev_upload(tr, h.slot, &p, s))) return rc;
+  d.slot = p ? p : d.ptr;  // without any contribution: a valid (unused) array
+  if ((rc = dev_upload(tr, h.vid, &p, s))) return rc;
+  d.vid = p;
+  const double fl = (double)C * (double)h.slot.size();
+  const double by = 8.0 * fl + (double)d.n * (2.0 * kSplitSlices * split_kpad(h.nseg * C) + 4.0);
+  tr->steps.push_back({8, (int)tr->sums.size(), tr->cur_stage, fl, by});
+  tr->flops[tr->cur_stage] += fl;
+  tr->bytes[tr->cur_stage] += by;
+  tr->sums.push_back(d);
   return VP_OK;
 }
 
@@ -656,6 +695,12 @@ const double* table_ptr(const vp_tables_s* T, int t) {
 
 }  // namespace
 
+
+// Trees up to this many nodes launch their chain with programmatic dependent launch: CTAs that wait for the launch before
+// them keep near-field ones off their SMs, which costs more than the latency saved once the near field fills the chip.
+// Measured with / without: 64 leaves 93 / 111 us, 150,000 nodes 296 / 331 us, 10.5M nodes 7.02 / 6.78 ms; layers, whose
+// near part is small, 856 / 897 us (always on).
+constexpr long long kPdlNodes = 300000;
 
 int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   const vp_tables_s* T = tr->T;
@@ -716,22 +761,57 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   }
   l2t.M = 3 * n; l2t.K = E; l2t.lda = E; l2t.table = T_L2T; l2t.src = BUF_LOC; l2t.dst = BUF_USLOT; l2t.split_vec = 2;
   s2m.M = E; s2m.K = n; s2m.lda = n; s2m.table = T_S2M; s2m.src = BUF_F; s2m.dst = BUF_MP; s2m.split_vec = 0;
-  s2m.out_mode = 1;
+  // split precision: the upward pass works on slots too (leaf multipoles, and a contribution per child and channel),
+  // summed and sliced level by level; in FP64 BUF_MP and BUF_LOC hold the expansions themselves
+  const int Es = (E + 1) & ~1;
+  long long nup = 0;
+  std::vector<std::vector<long long>> upl(split ? (size_t)NB * nch : 0);
   for (long long i = 0; i < NB; ++i) {
     const Box& b = B[i];
     if (b.leaf < 0 || b.level < 2) continue;
     const long long slot = nus++;
     usl[i].push_back(slot * Us);
     l2t.entries.push_back({(long long)(b.level * T->l2t_stride_lvl()), i * E, slot * Us});
-    s2m.entries.push_back({(long long)(b.level * T->s2m_stride_lvl()), (long long)b.leaf * n, i * E});
+    s2m.entries.push_back({(long long)(b.level * T->s2m_stride_lvl()), (long long)b.leaf * n, split ? nup : i * E});
+    if (!split) continue;
+    for (int ch = 0; ch < nch; ++ch) upl[i * nch + ch].push_back(nup + ch * C);
+    nup += Es;
+  }
+  std::vector<HostGemm> up(split ? P.max_level + 1 : 0), down(up.size());
+  if (split) {
+    const long long mat = (long long)C * 4 * C, part = (long long)(T->levels + 1) * nch;
+    for (HostGemm& g : up) {
+      g.M = C; g.K = C; g.lda = 4 * C; g.table = T_M2M; g.src = BUF_MP; g.dst = BUF_MP; g.split_vec = 1;
+    }
+    for (HostGemm& g : down) {
+      g.M = C; g.K = C; g.lda = C; g.table = T_L2L; g.src = BUF_LOC; g.dst = BUF_LSLOT; g.split_vec = 3;
+    }
+    for (long long i = 0; i < NB; ++i) {
+      const int l = B[i].level;
+      for (int ch = 0; ch < nch; ++ch) {
+        if (B[i].leaf < 0 && l >= 2 && (ch || kact(l)))
+          for (int q = 0; q < 4; ++q, nup += Cs) {
+            up[l].entries.push_back({(q * part + (long long)l * nch + ch) * mat, (long long)(B[i].child0 + q) * E + ch * C, nup,
+                                     (long long)(B[i].child0 + q) * nch + ch});
+            upl[i * nch + ch].push_back(nup);
+          }
+        if (l >= 3 && (ch || kact(l - 1))) {
+          const int par = B[i].parent, q = (int)(i - B[par].child0);
+          const long long slot = nls++;
+          lsl[i * nch + ch].push_back(slot * Cs);
+          down[l].entries.push_back({(long long)((l - 1) * T->l2l_stride_lvl() + q * T->l2l_stride_q() + ch * T->l2l_stride_ch()),
+                                     (long long)par * E + ch * C, slot * Cs, (long long)par * nch + ch});
+        }
+      }
+    }
   }
   tr->n_lslot = nls;
   tr->n_uslot = nus;
 
   // ---- device buffers
-  TRY(cudaMalloc(&tr->mp, std::max<long long>(1, NB * E) * sizeof(double)));
+  TRY(cudaMalloc(&tr->mp, std::max<long long>(1, split ? nup : NB * E) * sizeof(double)));
   tr->allocs.push_back(tr->mp);
-  TRY(cudaMalloc(&tr->loc, std::max<long long>(1, NB * E) * sizeof(double)));
+  TRY(cudaMalloc(&tr->loc, std::max<long long>(1, split ? 1 : NB * E) * sizeof(double)));
   tr->allocs.push_back(tr->loc);
   TRY(cudaMalloc(&tr->lslot, std::max<long long>(1, nls * Cs) * sizeof(double)));
   tr->allocs.push_back(tr->lslot);
@@ -739,8 +819,8 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   tr->allocs.push_back(tr->uslot);
   if (split) {
     // sliced source vectors of every family
-    const long long nv[kVecFamilies] = {tr->n_leaves, NB * nch, NB, NB * nch, NB * nch, NB * nch};
-    const int kk[kVecFamilies] = {n, C, E, 2 * C, C, 2 * C};
+    const long long nv[kVecFamilies] = {tr->n_leaves, NB * nch, NB, NB * nch};
+    const int kk[kVecFamilies] = {n, C, E, C};
     for (int v = 0; v < kVecFamilies; ++v) {
       TRY(cudaMalloc(&tr->sv[v], std::max<long long>(1, nv[v] * kSplitSlices * split_kpad(kk[v])) * 2));
       tr->allocs.push_back(tr->sv[v]);
@@ -751,52 +831,85 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
 
   int rc;
   // ---- steps, in pass order
+  auto add_out = [&]() {
+    HostReduce r;
+    r.M = 3 * n; r.final_out = 1; r.src = BUF_USLOT;
+    r.ptr.push_back(0);
+    for (int k = 0; k < tr->n_leaves; ++k) {
+      const int bi = P.leaf_box[k];
+      r.dst_off.push_back((long long)k * n);
+      for (long long o : usl[bi]) r.slot.push_back(o);
+      r.ptr.push_back((long long)r.slot.size());
+    }
+    return upload_reduce(tr, r, s);
+  };
+  if (split) {
+    std::vector<long long> lvl(P.max_level + 2, NB);  // first box of each level (boxes are listed by level)
+    for (long long i = NB - 1; i >= 0; --i) lvl[B[i].level] = i;
+    // multipoles (family 1) of a level, locals (family 3) of its internal boxes
+    auto add_sum = [&](int l, bool upward) {
+      HostSum h;
+      h.family = upward ? 1 : 3;
+      h.buf = upward ? BUF_MP : BUF_LSLOT;
+      for (long long i = lvl[l]; i < lvl[l + 1]; ++i)
+        for (int ch = 0; ch < nch; ++ch) {
+          if (!upward && (B[i].leaf >= 0 || !(ch || kact(l)))) continue;
+          h.segment((upward ? upl : lsl)[i * nch + ch]);
+          h.vid.push_back(i * nch + ch);
+        }
+      return upload_sum(tr, h, s);
+    };
+    tr->pdl = tr->N <= kPdlNodes;
+    tr->cur_stage = VP_STAGE_UPWARD;
+    if ((rc = add_slice(tr, 0, BUF_F, n, n, 0, n, tr->n_leaves, nullptr, nullptr, s))) return rc;
+    if ((rc = upload_gemm(tr, s2m, s))) return rc;
+    for (int l = P.max_level; l >= 2; --l) {
+      if ((rc = upload_gemm(tr, up[l], s))) return rc;  // children of level l (none at the deepest)
+      if ((rc = add_sum(l, true))) return rc;
+    }
+    tr->cur_stage = VP_STAGE_M2L;
+    if ((rc = upload_gemm(tr, m2l, s))) return rc;
+    if ((rc = upload_gemm(tr, s2l, s))) return rc;
+    tr->cur_stage = VP_STAGE_DOWNWARD;
+    for (int l = 2; l <= P.max_level; ++l) {
+      if ((rc = upload_gemm(tr, down[l], s))) return rc;  // parents of level l (none at level 2)
+      if ((rc = add_sum(l, false))) return rc;
+    }
+    tr->cur_stage = VP_STAGE_TARGETS;
+    HostSum h;  // locals of leaves, both channels together
+    h.family = 2; h.buf = BUF_LSLOT; h.nseg = nch;
+    for (long long i = 0; i < NB; ++i) {
+      if (B[i].leaf < 0 || B[i].level < 2) continue;
+      for (int ch = 0; ch < nch; ++ch) h.segment(lsl[i * nch + ch]);
+      h.vid.push_back(i);
+    }
+    if ((rc = upload_sum(tr, h, s))) return rc;
+    if ((rc = upload_gemm(tr, l2t, s))) return rc;
+    if ((rc = upload_gemm(tr, m2t, s))) return rc;
+    tr->cur_stage = VP_STAGE_NEAR;
+    if ((rc = upload_gemm(tr, nearg, s))) return rc;
+    tr->cur_stage = VP_STAGE_OUTPUT;
+    return add_out();
+  }
   tr->cur_stage = VP_STAGE_UPWARD;
   tr->steps.push_back({2, 0, tr->cur_stage, 0.0, 8.0 * (double)NB * E});  // clear multipoles
   tr->bytes[tr->cur_stage] += 8.0 * (double)NB * E;
-  if (split && (rc = add_slice(tr, 0, BUF_F, n, n, 0, n, tr->n_leaves, nullptr, nullptr, s))) return rc;
   if ((rc = upload_gemm(tr, s2m, s))) return rc;
   for (int l = P.max_level - 1; l >= 2; --l) {
-    if (!split) {
-      HostGemm m2m;
-      m2m.M = C; m2m.K = 4 * C; m2m.kseg = C; m2m.seg_stride = E; m2m.lda = 4 * C; m2m.table = T_M2M;
-      m2m.src = BUF_MP; m2m.dst = BUF_MP;
-      for (long long i = 0; i < NB; ++i) {
-        if (B[i].level != l || B[i].leaf >= 0) continue;
-        for (int ch = 0; ch < nch; ++ch) {
-          if (ch == 0 && !kact(l)) continue;
-          m2m.entries.push_back({(long long)(l * T->m2m_stride_lvl() + ch * T->m2m_stride_ch()),
-                                 (long long)B[i].child0 * E + ch * C, i * E + ch * C});
-        }
+    HostGemm m2m;
+    m2m.M = C; m2m.K = 4 * C; m2m.kseg = C; m2m.seg_stride = E; m2m.lda = 4 * C; m2m.table = T_M2M;
+    m2m.src = BUF_MP; m2m.dst = BUF_MP;
+    for (long long i = 0; i < NB; ++i) {
+      if (B[i].level != l || B[i].leaf >= 0) continue;
+      for (int ch = 0; ch < nch; ++ch) {
+        if (ch == 0 && !kact(l)) continue;
+        m2m.entries.push_back({(long long)(l * T->m2m_stride_lvl() + ch * T->m2m_stride_ch()),
+                               (long long)B[i].child0 * E + ch * C, i * E + ch * C});
       }
-      if ((rc = upload_gemm(tr, m2m, s))) return rc;
-      continue;
     }
-    // split precision: children 0-1 (overwrite) then children 2-3 (accumulate), K = 2C each
-    for (int half = 0; half < 2; ++half) {
-      HostGemm m2m;
-      m2m.M = C; m2m.K = 2 * C; m2m.kseg = C; m2m.seg_stride = E; m2m.lda = 4 * C;
-      m2m.table = half ? T_M2M_HI : T_M2M_LO;
-      m2m.src = BUF_MP; m2m.dst = BUF_MP; m2m.split_vec = half ? 5 : 3; m2m.out_mode = half ? 2 : 1;
-      std::vector<long long> sbase, svid;
-      for (long long i = 0; i < NB; ++i) {
-        if (B[i].level != l || B[i].leaf >= 0) continue;
-        for (int ch = 0; ch < nch; ++ch) {
-          if (ch == 0 && !kact(l)) continue;
-          const long long src = (long long)(B[i].child0 + 2 * half) * E + ch * C;
-          m2m.entries.push_back({(long long)(l * T->m2m_stride_lvl() + ch * T->m2m_stride_ch()), src,
-                                 i * E + ch * C, i * nch + ch});
-          sbase.push_back(src);
-          svid.push_back(i * nch + ch);
-        }
-      }
-      if ((rc = add_slice(tr, half ? 5 : 3, BUF_MP, 2 * C, C, E, 0, (long long)svid.size(), &sbase, &svid, s)))
-        return rc;
-      if ((rc = upload_gemm(tr, m2m, s))) return rc;
-    }
+    if ((rc = upload_gemm(tr, m2m, s))) return rc;
   }
   tr->cur_stage = VP_STAGE_M2L;
-  if (split && (rc = add_slice(tr, 1, BUF_MP, C, C, 0, C, NB * nch, nullptr, nullptr, s))) return rc;
   if ((rc = upload_gemm(tr, m2l, s))) return rc;
   if ((rc = upload_gemm(tr, s2l, s))) return rc;
   tr->cur_stage = VP_STAGE_DOWNWARD;
@@ -817,8 +930,6 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   for (int l = 3; l <= P.max_level; ++l) {
     HostGemm l2l;
     l2l.M = C; l2l.K = C; l2l.lda = C; l2l.accumulate = 1; l2l.table = T_L2L; l2l.src = BUF_LOC; l2l.dst = BUF_LOC;
-    l2l.split_vec = 4; l2l.out_mode = 2;
-    std::vector<long long> sbase, svid;
     for (long long i = 0; i < NB; ++i) {
       if (B[i].level != l) continue;
       const int par = B[i].parent;
@@ -826,36 +937,18 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
       for (int ch = 0; ch < nch; ++ch) {
         if (ch == 0 && !kact(l - 1)) continue;
         l2l.entries.push_back({(long long)((l - 1) * T->l2l_stride_lvl() + q * T->l2l_stride_q() + ch * T->l2l_stride_ch()),
-                               (long long)par * E + ch * C, i * E + ch * C, (long long)par * nch + ch});
-        if (q == 0) {  // each parent's local is sliced once
-          sbase.push_back((long long)par * E + ch * C);
-          svid.push_back((long long)par * nch + ch);
-        }
+                               (long long)par * E + ch * C, i * E + ch * C});
       }
     }
-    if (split && (rc = add_slice(tr, 4, BUF_LOC, C, C, 0, 0, (long long)svid.size(), &sbase, &svid, s))) return rc;
     if ((rc = upload_gemm(tr, l2l, s))) return rc;
   }
   tr->cur_stage = VP_STAGE_TARGETS;
-  if (split && (rc = add_slice(tr, 2, BUF_LOC, E, E, 0, E, NB, nullptr, nullptr, s))) return rc;
   if ((rc = upload_gemm(tr, l2t, s))) return rc;
   if ((rc = upload_gemm(tr, m2t, s))) return rc;
   tr->cur_stage = VP_STAGE_NEAR;
   if ((rc = upload_gemm(tr, nearg, s))) return rc;
   tr->cur_stage = VP_STAGE_OUTPUT;
-  {
-    HostReduce r;
-    r.M = 3 * n; r.final_out = 1; r.src = BUF_USLOT;
-    r.ptr.push_back(0);
-    for (int k = 0; k < tr->n_leaves; ++k) {
-      const int bi = P.leaf_box[k];
-      r.dst_off.push_back((long long)k * n);
-      for (long long o : usl[bi]) r.slot.push_back(o);
-      r.ptr.push_back((long long)r.slot.size());
-    }
-    if ((rc = upload_reduce(tr, r, s))) return rc;
-  }
-  return VP_OK;
+  return add_out();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -926,6 +1019,11 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
   std::vector<std::vector<long long>> lsl((size_t)NC * NB * nch), usl((size_t)NC * NB);
   long long nls = 0, nus = 0;
 
+  // split precision: slots in the upward pass too (see build_tree)
+  const bool split = T->precision == VP_PREC_SPLIT;
+  const int Es = (E + 1) & ~1;
+  long long nup = 0;
+  std::vector<std::vector<long long>> upl(split ? (size_t)NC * NB * nch : 0);
   std::vector<PtInst> ps2m, ps2l, pnear;
   for (long long i = 0; i < NB; ++i) {
     const Box& b = B[i];
@@ -933,8 +1031,11 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
     const double h = T->h(b.level), r = h / std::sqrt(2.0);
     PtInst I{};
     I.cx = x0 + (b.ix + 0.5) * h; I.cy = y0 + (b.iy + 0.5) * h; I.R = 1.25 * r; I.r = r;
-    I.j0 = bins.first[i]; I.ns = bins.count[i]; I.kact = kact(b.level); I.dst = off(0, i);
+    I.j0 = bins.first[i]; I.ns = bins.count[i]; I.kact = kact(b.level); I.dst = split ? nup : off(0, i);
     ps2m.push_back(I);
+    if (!split) continue;
+    for (int a = 0; a < NC; ++a, nup += Es)
+      for (int ch = 0; ch < nch; ++ch) upl[(size_t)(a * NB + i) * nch + ch].push_back(nup + ch * C);
   }
   HostGemm m2l, l2t, m2t;
   m2l.M = C; m2l.K = C; m2l.lda = C; m2l.table = T_M2L; m2l.src = BUF_MP; m2l.dst = BUF_LSLOT; m2l.split_vec = 1;
@@ -1000,23 +1101,54 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
     I.j0 = bins.first[u.src]; I.ns = bins.count[u.src]; I.kact = 1; I.dst = base * Us;
     pnear.push_back(I);
   }
+  std::vector<HostGemm> up(split ? P.max_level + 1 : 0), down(up.size());
+  if (split) {
+    const long long mat = (long long)C * 4 * C, part = (long long)(T->levels + 1) * nch;
+    for (HostGemm& g : up) {
+      g.M = C; g.K = C; g.lda = 4 * C; g.table = T_M2M; g.src = BUF_MP; g.dst = BUF_MP; g.split_vec = 1;
+    }
+    for (HostGemm& g : down) {
+      g.M = C; g.K = C; g.lda = C; g.table = T_L2L; g.src = BUF_LOC; g.dst = BUF_LSLOT; g.split_vec = 3;
+    }
+    for (int a = 0; a < NC; ++a)
+      for (long long i = 0; i < NB; ++i) {
+        const int l = B[i].level;
+        for (int ch = 0; ch < nch; ++ch) {
+          if (B[i].leaf < 0 && has[i] && l >= 2 && (ch || kact(l)))
+            for (int q = 0; q < 4; ++q) {
+              const long long c = B[i].child0 + q;
+              if (!has[c]) continue;
+              up[l].entries.push_back({(q * part + (long long)l * nch + ch) * mat, off(a, c) + ch * C, nup,
+                                       (a * NB + c) * nch + ch});
+              upl[(size_t)(a * NB + i) * nch + ch].push_back(nup);
+              nup += Cs;
+            }
+          if (l >= 3 && (ch || kact(l - 1))) {
+            const int par = B[i].parent, q = (int)(i - B[par].child0);
+            const long long slot = nls++;
+            lsl[(size_t)(a * NB + i) * nch + ch].push_back(slot * Cs);
+            down[l].entries.push_back({(long long)((l - 1) * T->l2l_stride_lvl() + q * T->l2l_stride_q() + ch * T->l2l_stride_ch()),
+                                       off(a, par) + ch * C, slot * Cs, (a * NB + par) * nch + ch});
+          }
+        }
+      }
+  }
   tr->n_lslot = nls;
   tr->n_uslot = nus;
 
   // ---- device buffers
   tr->mp_elems = NC * NB * E;
-  TRY(cudaMalloc(&tr->mp, std::max<long long>(1, NC * NB * E) * sizeof(double)));
+  TRY(cudaMalloc(&tr->mp, std::max<long long>(1, split ? nup : NC * NB * E) * sizeof(double)));
   tr->allocs.push_back(tr->mp);
-  TRY(cudaMalloc(&tr->loc, std::max<long long>(1, NC * NB * E) * sizeof(double)));
+  TRY(cudaMalloc(&tr->loc, std::max<long long>(1, split ? 1 : NC * NB * E) * sizeof(double)));
   tr->allocs.push_back(tr->loc);
   TRY(cudaMalloc(&tr->lslot, std::max<long long>(1, nls * Cs) * sizeof(double)));
   tr->allocs.push_back(tr->lslot);
   TRY(cudaMalloc(&tr->uslot, std::max<long long>(1, nus * Us) * sizeof(double)));
   tr->allocs.push_back(tr->uslot);
-  const bool split = T->precision == VP_PREC_SPLIT;
   if (split) {
-    const long long nv[kVecFamilies] = {1, NC * NB * nch, NC * NB, NC * NB * nch, NC * NB * nch, NC * NB * nch};
-    const int kk[kVecFamilies] = {n, C, E, 2 * C, C, 2 * C};
+    const long long nv[kVecFamilies] = {1, NC * NB * nch, NC * NB, NC * NB * nch};
+    const int kk[kVecFamilies] = {n, C, E, C};
     for (int v = 0; v < kVecFamilies; ++v) {
       TRY(cudaMalloc(&tr->sv[v], std::max<long long>(1, nv[v] * kSplitSlices * split_kpad(kk[v])) * 2));
       tr->allocs.push_back(tr->sv[v]);
@@ -1026,12 +1158,57 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
   }
 
   int rc;
+  if (split) {
+    std::vector<std::vector<long long>> at(P.max_level + 1);  // boxes of each level
+    for (long long i = 0; i < NB; ++i) at[B[i].level].push_back(i);
+    // multipoles (family 1) of the boxes with sources of a level, locals (family 3) of its internal boxes
+    auto add_sum = [&](int l, bool upward) {
+      HostSum h;
+      h.family = upward ? 1 : 3;
+      h.buf = upward ? BUF_MP : BUF_LSLOT;
+      for (int a = 0; a < NC; ++a)
+        for (long long i : at[l])
+          for (int ch = 0; ch < nch; ++ch) {
+            if (upward ? !has[i] : (B[i].leaf >= 0 || !(ch || kact(l)))) continue;
+            h.segment((upward ? upl : lsl)[(size_t)(a * NB + i) * nch + ch]);
+            h.vid.push_back((a * NB + i) * nch + ch);
+          }
+      return upload_sum(tr, h, s);
+    };
+    tr->pdl = true;
+    tr->cur_stage = VP_STAGE_UPWARD;
+    if ((rc = upload_pt(tr, ps2m, 2 * E, E, Es, BUF_MP, 0, S, s))) return rc;
+    for (int l = P.max_level; l >= 2; --l) {
+      if ((rc = upload_gemm(tr, up[l], s))) return rc;
+      if ((rc = add_sum(l, true))) return rc;
+    }
+    tr->cur_stage = VP_STAGE_M2L;
+    if ((rc = upload_gemm(tr, m2l, s))) return rc;
+    if ((rc = upload_pt(tr, ps2l, 2 * E, C, Cs, BUF_LSLOT, 1, S, s))) return rc;
+    tr->cur_stage = VP_STAGE_DOWNWARD;
+    for (int l = 2; l <= P.max_level; ++l) {
+      if ((rc = upload_gemm(tr, down[l], s))) return rc;
+      if ((rc = add_sum(l, false))) return rc;
+    }
+    tr->cur_stage = VP_STAGE_TARGETS;
+    HostSum h;
+    h.family = 2; h.buf = BUF_LSLOT; h.nseg = nch;
+    for (int a = 0; a < NC; ++a)
+      for (long long i = 0; i < NB; ++i) {
+        if (B[i].leaf < 0 || B[i].level < 2) continue;
+        for (int ch = 0; ch < nch; ++ch) h.segment(lsl[(size_t)(a * NB + i) * nch + ch]);
+        h.vid.push_back(a * NB + i);
+      }
+    if ((rc = upload_sum(tr, h, s))) return rc;
+    if ((rc = upload_gemm(tr, l2t, s))) return rc;
+    if ((rc = upload_gemm(tr, m2t, s))) return rc;
+  } else {
   tr->cur_stage = VP_STAGE_UPWARD;
   tr->steps.push_back({2, 0, tr->cur_stage, 0.0, 8.0 * (double)(NC * NB * E)});
   tr->bytes[tr->cur_stage] += 8.0 * (double)(NC * NB * E);
   if ((rc = upload_pt(tr, ps2m, 2 * E, E, NB * E, BUF_MP, 0, S, s))) return rc;
   for (int l = P.max_level - 1; l >= 2; --l) {
-    if (!split) {
+    {
       HostGemm m2m;
       m2m.M = C; m2m.K = 4 * C; m2m.kseg = C; m2m.seg_stride = E; m2m.lda = 4 * C; m2m.table = T_M2M;
       m2m.src = BUF_MP; m2m.dst = BUF_MP;
@@ -1045,34 +1222,9 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
           }
       }
       if ((rc = upload_gemm(tr, m2m, s))) return rc;
-      continue;
-    }
-    for (int half = 0; half < 2; ++half) {
-      HostGemm m2m;
-      m2m.M = C; m2m.K = 2 * C; m2m.kseg = C; m2m.seg_stride = E; m2m.lda = 4 * C;
-      m2m.table = half ? T_M2M_HI : T_M2M_LO;
-      m2m.src = BUF_MP; m2m.dst = BUF_MP; m2m.split_vec = half ? 5 : 3; m2m.out_mode = half ? 2 : 1;
-      std::vector<long long> sbase, svid;
-      for (long long i = 0; i < NB; ++i) {
-        if (B[i].level != l || B[i].leaf >= 0 || !has[i]) continue;
-        for (int a = 0; a < NC; ++a)
-          for (int ch = 0; ch < nch; ++ch) {
-            if (ch == 0 && !kact(l)) continue;
-            const long long src = off(a, B[i].child0 + 2 * half) + ch * C;
-            const long long vid = (a * NB + i) * nch + ch;
-            m2m.entries.push_back({(long long)(l * T->m2m_stride_lvl() + ch * T->m2m_stride_ch()), src,
-                                   off(a, i) + ch * C, vid});
-            sbase.push_back(src);
-            svid.push_back(vid);
-          }
-      }
-      if ((rc = add_slice(tr, half ? 5 : 3, BUF_MP, 2 * C, C, E, 0, (long long)svid.size(), &sbase, &svid, s)))
-        return rc;
-      if ((rc = upload_gemm(tr, m2m, s))) return rc;
     }
   }
   tr->cur_stage = VP_STAGE_M2L;
-  if (split && (rc = add_slice(tr, 1, BUF_MP, C, C, 0, C, NC * NB * nch, nullptr, nullptr, s))) return rc;
   if ((rc = upload_gemm(tr, m2l, s))) return rc;
   if ((rc = upload_pt(tr, ps2l, 2 * E, C, Cs, BUF_LSLOT, 1, S, s))) return rc;
   tr->cur_stage = VP_STAGE_DOWNWARD;
@@ -1094,8 +1246,6 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
   for (int l = 3; l <= P.max_level; ++l) {
     HostGemm l2l;
     l2l.M = C; l2l.K = C; l2l.lda = C; l2l.accumulate = 1; l2l.table = T_L2L; l2l.src = BUF_LOC; l2l.dst = BUF_LOC;
-    l2l.split_vec = 4; l2l.out_mode = 2;
-    std::vector<long long> sbase, svid;
     for (long long i = 0; i < NB; ++i) {
       if (B[i].level != l) continue;
       const int par = B[i].parent;
@@ -1103,22 +1253,16 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
       for (int a = 0; a < NC; ++a)
         for (int ch = 0; ch < nch; ++ch) {
           if (ch == 0 && !kact(l - 1)) continue;
-          const long long vid = (a * NB + par) * nch + ch;
           l2l.entries.push_back({(long long)((l - 1) * T->l2l_stride_lvl() + q * T->l2l_stride_q() + ch * T->l2l_stride_ch()),
-                                 off(a, par) + ch * C, off(a, i) + ch * C, vid});
-          if (q == 0) {
-            sbase.push_back(off(a, par) + ch * C);
-            svid.push_back(vid);
-          }
+                                 off(a, par) + ch * C, off(a, i) + ch * C});
         }
     }
-    if (split && (rc = add_slice(tr, 4, BUF_LOC, C, C, 0, 0, (long long)svid.size(), &sbase, &svid, s))) return rc;
     if ((rc = upload_gemm(tr, l2l, s))) return rc;
   }
   tr->cur_stage = VP_STAGE_TARGETS;
-  if (split && (rc = add_slice(tr, 2, BUF_LOC, E, E, 0, E, NC * NB, nullptr, nullptr, s))) return rc;
   if ((rc = upload_gemm(tr, l2t, s))) return rc;
   if ((rc = upload_gemm(tr, m2t, s))) return rc;
+  }
   tr->cur_stage = VP_STAGE_NEAR;
   if ((rc = upload_pt(tr, pnear, 2 * n, n, Us, BUF_USLOT, 2, S, s))) return rc;
   tr->cur_stage = VP_STAGE_OUTPUT;
@@ -1143,7 +1287,7 @@ SplitArgs split_args(const vp_tree_s* tr, const DevSplit& d, double* const* bufs
   const SplitTables* stt = static_cast<const SplitTables*>(tr->T->near_split);
   const SplitTable* tb = d.table == T_NEAR ? &stt->near : d.table == T_S2M ? &stt->s2m : d.table == T_L2T
                          ? &stt->l2t : d.table == T_M2L ? &stt->m2l : d.table == T_M2T ? &stt->m2t
-                         : d.table == T_M2M_LO ? &stt->m2m_lo : d.table == T_M2M_HI ? &stt->m2m_hi
+                         : d.table == T_M2M ? &stt->m2m
                          : d.table == T_L2L ? &stt->l2l : &stt->s2l;
   SplitArgs a = d.args;
   a.A = static_cast<const slice_t*>(tb->A);
@@ -1152,7 +1296,7 @@ SplitArgs split_args(const vp_tree_s* tr, const DevSplit& d, double* const* bufs
   a.ea_ld = tb->M;
   a.B = static_cast<const slice_t*>(tr->sv[d.vec]);
   a.eb = tr->se[d.vec];
-  a.Y = bufs[d.dst];
+  a.Y = reinterpret_cast<float2*>(bufs[d.dst]);
   a.tiles = d.tiles[d.engine];
   return a;
 }
@@ -1172,7 +1316,7 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
   double* bufs[BUF_COUNT] = {nullptr, tr->mp, tr->loc, tr->lslot, tr->uslot};
   const bool overlap = !ev && !step_ev && tr->side;
   int step_no = 0;
-  bool src_ready = false, near_started = false, joined = !overlap;
+  bool src_ready = false, near_started = false, joined = !overlap, after_kernel = false;
   if (overlap) {
     TRY(cudaEventRecord(tr->ev_fork, s0));
     TRY(cudaStreamWaitEvent(tr->side, tr->ev_fork, 0));
@@ -1194,6 +1338,9 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
       near_started = true;
     }
     const cudaStream_t s = (!overlap || near_step || st.stage == VP_STAGE_OUTPUT) ? s0 : tr->side;
+    // a launch of the chain may start while the one before it ends, unless an event lies between them
+    const bool pdl = tr->pdl && after_kernel && s == tr->side;
+    if (s == tr->side) after_kernel = overlap && st.kind != 2;
     if (st.kind == 2) {
       const long long elems = tr->mp_elems ? tr->mp_elems : (long long)tr->n_boxes * T->E;
       TRY(cudaMemsetAsync(tr->mp, 0, (size_t)elems * sizeof(double), s));
@@ -1220,24 +1367,25 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
       if (rc) return rc;
     } else if (st.kind == 6) {
       const DevPt& d = tr->pts[st.index];
-      // slots of split-precision trees hold double-float values; multipole coefficients are FP64
-      const int df = T->precision == VP_PREC_SPLIT && d.dst != BUF_MP;
+      // slots of split-precision trees hold double-float values
+      const int df = T->precision == VP_PREC_SPLIT;
       const int rc = launch_pt_apply(d.rows, d.rb, d.bs, df, d.inst, d.n_inst, tr->d_perm, bufs_c[BUF_F], d.A,
                                      bufs[d.dst], s);
       if (rc) return rc;
     } else if (st.kind == 3) {
       const DevSlice& d = tr->slice_ops[st.index];
       const int rc = launch_slice_list(bufs_c[d.buf], d.base, d.vid, d.n, d.K, d.kseg, d.seg_stride, d.cstride,
-                                       tr->sv[d.family], tr->se[d.family], s);
+                                       tr->sv[d.family], tr->se[d.family], s, pdl);
       if (rc) return rc;
       if (overlap && d.family == 0 && !near_started) {
         TRY(cudaEventRecord(tr->ev_src, s));
         src_ready = true;
+        after_kernel = false;
       }
     } else if (st.kind == 4) {
       const DevSplit& d = tr->splits[st.index];
       SplitArgs a = split_args(tr, d, bufs);
-      const int rc = launch_split_gemm(a, d.n_tiles[d.engine], s, d.engine, near_step ? 1 : 0);
+      const int rc = launch_split_gemm(a, d.n_tiles[d.engine], s, d.engine, near_step ? 1 : 0, pdl);
       if (rc) return rc;
     } else if (st.kind == 5) {
       const DevReduce& d = tr->reduces[st.index];
@@ -1246,7 +1394,12 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
       a.dst_off = d.args.dst_off; a.ptr = d.args.ptr; a.slot = d.args.slot;
       a.S = bufs_c[d.src];
       if (a.final_out) { a.u = u; a.g = g; } else { a.Y = bufs[d.dst]; }
-      const int rc = launch_reduce_df(a, d.n_dst, s);
+      const int rc = launch_reduce_df(a, d.n_dst, s, pdl);
+      if (rc) return rc;
+    } else if (st.kind == 8) {
+      const DevSum& d = tr->sums[st.index];
+      const int rc = launch_sum_slice(T->C, d.nseg, d.n, d.ptr, d.slot, d.vid, bufs[d.buf], tr->sv[d.family],
+                                      tr->se[d.family], s, pdl);
       if (rc) return rc;
     }
   }

@@ -102,39 +102,12 @@ __global__ void k_slice_rows(const double* __restrict__ A, long long mstride, in
   if (lane == 0) ea[mat * M + r] = e;
 }
 
-// Slice a list of vectors. Vector v (v < nlist) has identifier id = vid ? vid[v] : v and elements
-// x_k = X[b + (k / kseg) * seg_stride + k % kseg], k < K <= 2 kseg, b = base ? base[v] : v * cstride;
-// output out[id][Kpad / 16][s][16] (the S slices of each K step of 16 are contiguous, so one
-// column of a K step is one 32 S-byte block for the GEMM engines' gathers) and eb[id].
-//
-// L lanes per vector (a power of two, L >= Kpad / 8), a lane taking 8 consecutive elements: they are read once and
-// kept for the digits, and a slice of them is one 16-byte store (2-byte stores, six per element, and a second
-// read of the vector took 571 us an evaluation of the full-size star, now 459). The digits are those of digits(): with 128 added to each of the lower five,
-// balanced digits are plain bytes, and a byte under the bits of 2^23 is a float that one multiply-add turns into
-// (byte - 128) 2^(-8 (i + 1)), exact. Measured: the star's leaf sources (40,897 vectors of 256) 79 -> 52 us = 4.0 TB/s.
+// The S digits (digits()) of 8 consecutive elements with the vector's exponent e, one 16-byte store per slice. With 128
+// added to each of the lower five, balanced digits are plain bytes, and a byte under the bits of 2^23 is a float
+// that one multiply-add turns into (byte - 128) 2^(-8 (i + 1)), exact.
 template <int S>
-__global__ void __launch_bounds__(256) k_slice_list(const double* __restrict__ X, const long long* __restrict__ base,
-                                                    const long long* __restrict__ vid, long long nlist, int K, int kseg,
-                                                    long long seg_stride, long long cstride, int Kpad, int lg_l,
-                                                    slice_t* __restrict__ out, int* __restrict__ eb) {
+__device__ inline void store_digits(const double (&x)[8], int e, slice_t* o) {
   static_assert(S == 6, "five balanced bytes and a leading digit");
-  const int L = 1 << lg_l, l = threadIdx.x & (L - 1);
-  const long long v = (blockIdx.x * 256ll + threadIdx.x) >> lg_l;
-  const bool ok = v < nlist;
-  const long long b = !ok ? 0 : (base ? base[v] : v * cstride);
-  double x[8];
-  double mx = 0.0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int k = 8 * l + i;
-    x[i] = ok && k < K ? X[b + k + (k >= kseg ? seg_stride - kseg : 0)] : 0.0;
-    mx = fmax(mx, fabs(x[i]));
-  }
-  for (int o = L >> 1; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (!ok || 8 * l >= Kpad) return;
-  const int e = exponent_of(mx);
-  const long long id = vid ? vid[v] : v;
-  if (l == 0) eb[id] = e;
   unsigned w[S][4];
 #pragma unroll
   for (int i = 0; i < 8; i += 2) {
@@ -165,9 +138,44 @@ __global__ void __launch_bounds__(256) k_slice_list(const double* __restrict__ X
       w[d][i >> 1] = *reinterpret_cast<const unsigned*>(&p) ^ sign;
     }
   }
-  slice_t* o = out + id * (long long)S * Kpad + (l >> 1) * (S * 16) + (l & 1) * 8;
 #pragma unroll
   for (int d = 0; d < S; ++d) *reinterpret_cast<uint4*>(o + d * 16) = make_uint4(w[d][0], w[d][1], w[d][2], w[d][3]);
+}
+
+// Slice a list of vectors. Vector v (v < nlist) has identifier id = vid ? vid[v] : v and elements
+// x_k = X[b + (k / kseg) * seg_stride + k % kseg], k < K <= 2 kseg, b = base ? base[v] : v * cstride;
+// output out[id][Kpad / 16][s][16] (the S slices of each K step of 16 are contiguous, so one
+// column of a K step is one 32 S-byte block for the GEMM engines' gathers) and eb[id].
+//
+// L lanes per vector (a power of two, L >= Kpad / 8), a lane taking 8 consecutive elements: they are read once and
+// kept for the digits, and a slice of them is one 16-byte store (2-byte stores, six per element, and a second
+// read of the vector took 571 us an evaluation of the full-size star, now 459).
+// Measured: the star's leaf sources (40,897 vectors of 256) 79 -> 52 us = 4.0 TB/s.
+template <int S>
+__global__ void __launch_bounds__(256) k_slice_list(const double* __restrict__ X, const long long* __restrict__ base,
+                                                    const long long* __restrict__ vid, long long nlist, int K, int kseg,
+                                                    long long seg_stride, long long cstride, int Kpad, int lg_l,
+                                                    slice_t* __restrict__ out, int* __restrict__ eb) {
+  const int L = 1 << lg_l, l = threadIdx.x & (L - 1);
+  const long long v = (blockIdx.x * 256ll + threadIdx.x) >> lg_l;
+  const bool ok = v < nlist;
+  const long long b = !ok ? 0 : (base ? base[v] : v * cstride);
+  pdl_trigger();
+  pdl_wait();
+  double x[8];
+  double mx = 0.0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = 8 * l + i;
+    x[i] = ok && k < K ? X[b + k + (k >= kseg ? seg_stride - kseg : 0)] : 0.0;
+    mx = fmax(mx, fabs(x[i]));
+  }
+  for (int o = L >> 1; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (!ok || 8 * l >= Kpad) return;
+  const int e = exponent_of(mx);
+  const long long id = vid ? vid[v] : v;
+  if (l == 0) eb[id] = e;
+  store_digits<S>(x, e, out + id * (long long)S * Kpad + (l >> 1) * (S * 16) + (l & 1) * 8);
 }
 
 __device__ inline void df_add(float& hi, float& lo, float x) {
@@ -200,50 +208,17 @@ __device__ inline void fold4(float a0, float a1, float a2, float a3, float& h, f
   two_sum(s2, __fadd_rn(__fadd_rn(e, e2), a3), h, l);
 }
 
-// 2^e as a float / double (e in the normal range of the type).
+// 2^e as a float (e in its normal range).
 __device__ inline float pow2f(int e) { return __int_as_float((e + 127) << 23); }
-__device__ inline double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// One output element: double-float (h, l) times 2^e, as a double-float slot (out_mode 0) or in
-// FP64 (out_mode 1 overwrites, 2 adds to `old`, the value the destination held before the launch).
-// Scaling by a power of two is exact (ldexp only where 2^e itself is not a normal number). Callers
-// with out_mode 2 read the old values of a group of outputs first, so that the reads of the group
-// are in flight together instead of one read-add-store chain per element.
-// The 8 bytes store_out would write for out_mode 0 (double-float slot) or 1 (FP64), as a double.
-__device__ inline double out_value(const SplitArgs& a, float h, float l, int e) {
-  if (a.out_mode == 0) {
-    float2 o;
-    if (e >= -126 && e <= 127) {
-      const float sc = pow2f(e);
-      o.x = h * sc;
-      o.y = l * sc;
-    } else {
-      o.x = ldexpf(h, e);
-      o.y = ldexpf(l, e);
-    }
-    return __hiloint2double(__float_as_int(o.y), __float_as_int(o.x));
+// One output element: double-float (h, l) times 2^e as a double-float slot. Scaling by a power of two is exact (ldexp
+// only where 2^e itself is not a normal number).
+__device__ inline float2 out_value(float h, float l, int e) {
+  if (e >= -126 && e <= 127) {
+    const float sc = pow2f(e);
+    return make_float2(h * sc, l * sc);
   }
-  const double hl = (double)h + (double)l;
-  return (e >= -1022 && e <= 1023) ? hl * pow2d(e) : ldexp(hl, e);
-}
-
-__device__ inline void store_out(const SplitArgs& a, long long dst, int row, float h, float l, int e, double old) {
-  if (a.out_mode == 0) {
-    float2 o;
-    if (e >= -126 && e <= 127) {
-      const float sc = pow2f(e);
-      o.x = h * sc;
-      o.y = l * sc;
-    } else {
-      o.x = ldexpf(h, e);
-      o.y = ldexpf(l, e);
-    }
-    reinterpret_cast<float2*>(a.Y)[dst + row] = o;
-  } else {
-    const double hl = (double)h + (double)l;
-    const double val = (e >= -1022 && e <= 1023) ? hl * pow2d(e) : ldexp(hl, e);
-    reinterpret_cast<double*>(a.Y)[dst + row] = (a.out_mode == 2) ? old + val : val;
-  }
+  return make_float2(ldexpf(h, e), ldexpf(l, e));
 }
 
 __device__ inline void cp_async16(void* smem, const void* gmem, bool valid) {
@@ -284,6 +259,8 @@ __global__ void __launch_bounds__(BM * BN / 32) k_split_gemm(SplitArgs a) {
   slice_t* Bs = As + 2 * S * BM * kMPitch;                              // [2][S][BN][pitch]
   const SplitTile tile = a.tiles[blockIdx.x];
   const long long mat = a.a_mat[tile.group];
+  pdl_trigger();
+  pdl_wait();
   // this tile's rows in the tiled operator layout: [K step][slice][chunk][128 rows][8], rows from
   // m0 % 128 within the table tile
   const slice_t* Ag = a.A + (mat * a.nrt + (tile.m0 >> 7)) * (long long)(a.Kpad / 16) * S * 2048 + (tile.m0 & 127) * 8;
@@ -380,18 +357,6 @@ __global__ void __launch_bounds__(BM * BN / 32) k_split_gemm(SplitArgs a) {
       eb[cc] = cok[cc] ? a.eb[a.src_vec[tile.col0 + col]] : 0;
       dst[cc] = cok[cc] ? a.dst_off[tile.col0 + col] : 0;
     }
-    double old[2][2][2] = {};
-    if (a.out_mode == 2) {
-#pragma unroll
-      for (int cc = 0; cc < 2; ++cc)
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-          for (int rr = 0; rr < 2; ++rr) {
-            const int row = tile.m0 + wm * 32 + mt * 16 + gid + rr * 8;
-            if (cok[cc] && row < a.M) old[cc][mt][rr] = reinterpret_cast<const double*>(a.Y)[dst[cc] + row];
-          }
-    }
 #pragma unroll
     for (int cc = 0; cc < 2; ++cc) {
       if (!cok[cc]) continue;
@@ -404,7 +369,7 @@ __global__ void __launch_bounds__(BM * BN / 32) k_split_gemm(SplitArgs a) {
           float h, l;
           fold4(acc[0][mt][nt][rr * 2 + cc], acc[1][mt][nt][rr * 2 + cc], acc[2][mt][nt][rr * 2 + cc],
                 acc[3][mt][nt][rr * 2 + cc], h, l);
-          store_out(a, dst[cc], row, h, l, ea[row] + eb[cc], old[cc][mt][rr]);
+          a.Y[dst[cc] + row] = out_value(h, l, ea[row] + eb[cc]);
         }
     }
   }
@@ -415,7 +380,7 @@ size_t mma_smem_bytes(int S, int BM, int BN) { return (size_t)2 * S * (BM + BN) 
 // ------------------------------------------------------------------ engine 1: tcgen05
 //
 // Persistent and warp-specialised: one CTA per SM walks the tile list (tile t, t + gridDim.x, ...).
-//  * warps 0-3 (producers) stage the operands of every K step of 16 into a 4-stage ring in the
+//  * warps 0-2 (producers) stage the operands of every K step of 16 into a 4-stage ring in the
 //    canonical K-major layout without swizzle (8-row x 16-byte core matrices): the operator slices
 //    (A), stored in that layout tile by tile, by one bulk copy (cp.async.bulk, 24 KB) issued by
 //    thread 0, whose bytes complete on the stage's `fullA` mbarrier (next core matrix along K 2048
@@ -426,11 +391,13 @@ size_t mma_smem_bytes(int S, int BM, int BN) { return (size_t)2 * S * (BM + BN) 
 //    tiles, so the next tile's operands stream in while the current one is drained. (Moving A by a
 //    tensor map whose boxes are 16 bytes wide -- the same layout built by the TMA unit -- made the
 //    whole K step 1.7x slower: narrow boxes cost the unit far more than one contiguous copy.)
-//  * warps 4 .. 15 (epilogue) read the accumulators (warp w: tensor-memory lanes 32 (w % 4) .. + 31,
-//    one accumulator row per thread, every third block of 16 columns), fold them in double-float and
-//    store. (Three warps per lane quadrant: the epilogue is the part of a tile that the MMAs wait
-//    for, and four producer warps issue a K step's copies easily.)
-//  * warp 16 (one thread) waits on `full`, fences the generic-proxy writes of the stage against the
+//  * warps 3 .. 18 (epilogue) read the accumulators (warp w: tensor-memory lanes 32 (w % 4) .. + 31, one accumulator row
+//    per thread, every fourth block of 8 columns, the next block's loads under the current one's fold), fold them
+//    in double-float and store. The epilogue is the part of a tile that the MMAs wait for, and a warp's chain of loads,
+//    folds and stores bounds it: measured on the full-size star, near / M2L / M2T launches with 12 warps and blocks of
+//    16 columns 2.54 / 1.43 / 0.67 ms, 16 warps 2.35 / 1.19 / 0.60, with the loads ahead 2.25 / 1.15 / 0.55 (near 0.70 of
+//    the bf16 peak). 20 warps keep 96 registers a thread: three producer warps issue a K step's copies as well as four.
+//  * warp 19 (one thread) waits on `full`, fences the generic-proxy writes of the stage against the
 //    async proxy, issues tcgen05.mma (kind::f16, bf16 operands, M = 128, N = BN, K = 16) into four
 //    fp32 accumulators in tensor memory (one per weight group) and commits to the stage's `empty`
 //    mbarrier; after a tile's last step it commits to `acc`, and it starts the next tile once the
@@ -441,11 +408,11 @@ size_t mma_smem_bytes(int S, int BM, int BN) { return (size_t)2 * S * (BM + BN) 
 
 __device__ int g_split_error = 0;
 
-constexpr int kTcProducers = 128;                 // warps 0-3
+constexpr int kTcProducers = 96;                  // warps 0-2
 #ifndef VP_TC_EPILOGUE_WARPS
-#define VP_TC_EPILOGUE_WARPS 12
+#define VP_TC_EPILOGUE_WARPS 16
 #endif
-constexpr int kTcEpilogue = 32 * VP_TC_EPILOGUE_WARPS;  // warps 8 .. 8 + warps - 1
+constexpr int kTcEpilogue = 32 * VP_TC_EPILOGUE_WARPS;  // warps 3 .. 18
 constexpr int kTcEpiParts = VP_TC_EPILOGUE_WARPS / 4;   // epilogue warps per tensor-memory lane quadrant
 constexpr int kTcMmaWarp = (kTcProducers + kTcEpilogue) / 32;
 constexpr int kTcThreads = kTcProducers + kTcEpilogue + 32;
@@ -454,7 +421,7 @@ constexpr int kTcStages = 4;
 constexpr int kTcCols = 512;                      // tensor-memory columns allocated per CTA
 constexpr int kTcA = kSplitBM * kTcKC;            // elements per A slice tile
 static_assert(kSplitBN[kEngineTcgen05] == 128 && kSplitBN[kEngineTcgen05N64] == 64, "tcgen05 tile widths");
-static_assert(kSplitBM == 128 && kTcProducers % 128 == 0 && kTcEpiParts * 128 == kTcEpilogue, "thread mapping");
+static_assert(kSplitBM == 128 && kTcProducers % 32 == 0 && kTcEpiParts * 128 == kTcEpilogue, "thread mapping");
 
 // Tile width BN (columns) of a tcgen05 engine: the four accumulators take 4 BN tensor-memory
 // columns, so at BN = 64 two sets fit and the MMAs of a tile run while the epilogue drains the
@@ -577,6 +544,23 @@ __device__ inline bool epi_all(bool pred) {
   return r != 0;
 }
 
+// Eight accumulator columns of the warp's lanes; valid after tmem_wait on them (whose operands order the uses).
+__device__ inline void tmem_ld8(unsigned taddr, float (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "r"(taddr));
+}
+__device__ inline void tmem_wait(float (&v)[kAcc][8]) {
+  static_assert(kAcc == 4, "32 registers");
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+f"(v[0][0]), "+f"(v[0][1]), "+f"(v[0][2]), "+f"(v[0][3]), "+f"(v[0][4]), "+f"(v[0][5]), "+f"(v[0][6]),
+                 "+f"(v[0][7]), "+f"(v[1][0]), "+f"(v[1][1]), "+f"(v[1][2]), "+f"(v[1][3]), "+f"(v[1][4]), "+f"(v[1][5]),
+                 "+f"(v[1][6]), "+f"(v[1][7]));
+  asm volatile("" : "+f"(v[2][0]), "+f"(v[2][1]), "+f"(v[2][2]), "+f"(v[2][3]), "+f"(v[2][4]), "+f"(v[2][5]), "+f"(v[2][6]),
+                    "+f"(v[2][7]), "+f"(v[3][0]), "+f"(v[3][1]), "+f"(v[3][2]), "+f"(v[3][3]), "+f"(v[3][4]), "+f"(v[3][5]),
+                    "+f"(v[3][6]), "+f"(v[3][7]));
+}
+
 // TR = 0: D [operator rows x columns] = operator slices (A) x gathered vectors (B), N = BN.
 // TR > 0 (operators of at most TR <= 128 rows, BN = 128): the transposed product D^T [columns x rows]
 // = gathered vectors (A, M = 128) x operator slices (B, N = TR), so every tensor-memory lane -- and
@@ -602,7 +586,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __shared__ int col_e[BN];
   // transposed tiles: per epilogue warp, eight outputs of its 32 lanes' destinations on their way to
   // coalesced stores
-  __shared__ __align__(16) double stage[TR ? kTcEpilogue / 32 : 1][32][8];
+  __shared__ __align__(16) float2 stage[TR ? kTcEpilogue / 32 : 1][32][8];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (warp == kTcMmaWarp) {
@@ -629,11 +613,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;\n");
   const unsigned tmem = tmem_base_sh;
   const int nk = a.Kpad / kTcKC;
+  pdl_trigger();
+  pdl_wait();
 
   if (warp < kTcProducers / 32) {
     // ---- producers: a K step of the gathered operand is BN columns x 2 S chunks of 16 bytes; a
     // column's chunks (slice, half) are contiguous in global memory, so consecutive threads take
-    // consecutive chunks: thread t copies chunks q = t + 128 i, i < kQ (column q / 2S, slice
+    // consecutive chunks: thread t copies chunks q = t + 96 i, i < kQ (column q / 2S, slice
     // (q % 2S) / 2, half q % 2)
     const slice_t* bsrc[kQ];
     int bdst[kQ];
@@ -687,207 +673,124 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         mbar_wait(&fullA[q % kTcStages], (unsigned)(q / kTcStages) & 1u);
     }
   } else if (warp < kTcMmaWarp) {
-    // ---- epilogue
-    if constexpr (TR > 0) {
-      // transposed tiles: lane = column of the tile (vector, destination), tensor-memory column =
-      // operator row
-      const int e = tid - kTcProducers;
-      const int q = warp & 3, part = (warp - kTcProducers / 32) >> 2;
-      int it = 0;
-      for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
-        const SplitTile tile = a.tiles[t];
-        for (int o = e; o < TR; o += kTcEpilogue) col_e[o] = o < a.M ? a.ea[a.a_mat[tile.group] * a.ea_ld + o] : 0;
-        const int pc = q * 32 + lane;
-        const bool pok = pc < tile.ncol;
-        const long long dst = pok ? a.dst_off[tile.col0 + pc] : 0;
-        const int ebv = pok ? a.eb[a.src_vec[tile.col0 + pc]] : 0;
-        const bool acc_ok = mbar_wait(&accbar[0], (unsigned)it & 1u, &abort_sh);
-        // uniform over the epilogue group (also publishes the row exponents written above)
-        if (!epi_all(acc_ok && !abort_sh)) {
-          abort_sh = 1;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;\n");
-#pragma unroll 1
-        for (int cb = part; cb < TR / 16; cb += kTcEpiParts) {
-          if (cb * 16 >= a.M) break;
-          float vv[kAcc][16];
-#pragma unroll
-          for (int w = 0; w < kAcc; ++w) {
-            const unsigned taddr = tmem + ((unsigned)(q * 32) << 16) + (unsigned)(w * TR + cb * 16);
-            unsigned rr[16];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];\n"
-                : "=r"(rr[0]), "=r"(rr[1]), "=r"(rr[2]), "=r"(rr[3]), "=r"(rr[4]), "=r"(rr[5]), "=r"(rr[6]),
-                  "=r"(rr[7]), "=r"(rr[8]), "=r"(rr[9]), "=r"(rr[10]), "=r"(rr[11]), "=r"(rr[12]), "=r"(rr[13]),
-                  "=r"(rr[14]), "=r"(rr[15])
-                : "r"(taddr));
-#pragma unroll
-            for (int cc = 0; cc < 16; ++cc) vv[w][cc] = __uint_as_float(rr[cc]);
-          }
-          asm volatile("tcgen05.wait::ld.sync.aligned;\n");
-          if (a.out_mode != 2 && cb * 16 + 16 <= a.M) {
-            // a full block of 16 outputs: each lane forms its 8-byte values (double-float slot or
-            // FP64), eight at a time, into the warp's staging rows; then lanes 8 g .. 8 g + 7 store
-            // eight consecutive outputs of destination 4 i + g, four destinations per instruction
-            double (*stg)[8] = stage[(warp - kTcProducers / 32)];
-#pragma unroll
-            for (int c8 = 0; c8 < 16; c8 += 8) {
-#pragma unroll
-              for (int cc = 0; cc < 8; ++cc) {
-                const int o = cb * 16 + c8 + cc;
-                float h, l;
-                fold4(vv[0][c8 + cc], vv[1][c8 + cc], vv[2][c8 + cc], vv[3][c8 + cc], h, l);
-                stg[lane][cc] = out_value(a, h, l, col_e[o] + ebv);
-              }
-              __syncwarp();
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const int src = 4 * i + (lane >> 3);
-                const long long d = __shfl_sync(0xffffffffu, dst, src);
-                if (q * 32 + src < tile.ncol)
-                  reinterpret_cast<double*>(a.Y)[d + cb * 16 + c8 + (lane & 7)] = stg[src][lane & 7];
-              }
-              __syncwarp();
-            }
-          } else if (pok && a.out_mode != 2) {
-#pragma unroll
-            for (int cc = 0; cc < 16; ++cc) {
-              const int o = cb * 16 + cc;
-              if (o >= a.M) break;
-              float h, l;
-              fold4(vv[0][cc], vv[1][cc], vv[2][cc], vv[3][cc], h, l);
-              store_out(a, dst, o, h, l, col_e[o] + ebv, 0.0);
-            }
-          } else if (pok) {
-            // accumulating launch: fold, read the old values of eight outputs together, store
-#pragma unroll
-            for (int cc = 0; cc < 16; ++cc) {
-              float h, l;
-              fold4(vv[0][cc], vv[1][cc], vv[2][cc], vv[3][cc], h, l);
-              vv[0][cc] = h;
-              vv[1][cc] = l;
-            }
-#pragma unroll
-            for (int c8 = 0; c8 < 16; c8 += 8) {
-              double old[8];
-#pragma unroll
-              for (int cc = 0; cc < 8; ++cc) {
-                const int o = cb * 16 + c8 + cc;
-                old[cc] = o < a.M ? reinterpret_cast<const double*>(a.Y)[dst + o] : 0.0;
-              }
-#pragma unroll
-              for (int cc = 0; cc < 8; ++cc) {
-                const int o = cb * 16 + c8 + cc;
-                if (o < a.M) store_out(a, dst, o, vv[0][c8 + cc], vv[1][c8 + cc], col_e[o] + ebv, old[cc]);
-              }
-            }
-          }
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;\n");
-        mbar_arrive(&tmem_free[0]);
-        asm volatile("bar.sync 1, %0;\n" ::"n"(kTcEpilogue) : "memory");
-      }
-    } else {
-
+    // ---- epilogue: warp w has tensor-memory lanes 32 (w % 4) .. + 31; the kTcEpiParts warps of a quadrant take its
+    // blocks of 8 accumulator columns in turn. The next block's loads run while this one is folded and stored, and
+    // tensor memory is handed back as soon as a warp's last block has been read.
     const int e = tid - kTcProducers;
-    // warp w reads tensor-memory lanes 32 (w % 4) .. + 31; the kTcEpiParts warps of a quadrant share
-    // its column blocks
     const int q = warp & 3, part = (warp - kTcProducers / 32) >> 2;
     int it = 0;
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
       const SplitTile tile = a.tiles[t];
       const int buf = it % kBufs;
-      if (e % (kTcEpilogue / BN) == 0) {
-        const int col = e / (kTcEpilogue / BN);
-        const bool cok = col < tile.ncol;
-        const long long v = cok ? a.src_vec[tile.col0 + col] : 0;
-        col_dst[col] = cok ? a.dst_off[tile.col0 + col] : 0;
-        col_e[col] = cok ? a.eb[v] : 0;
+      // normal tiles: lane = operator row, column = tile column (vector, destination); transposed tiles the other way
+      const int pos = q * 32 + lane;
+      long long dst = 0;
+      int own_e = 0, nblk;
+      bool ok;
+      if constexpr (TR > 0) {
+        for (int o = e; o < TR; o += kTcEpilogue) col_e[o] = o < a.M ? a.ea[a.a_mat[tile.group] * a.ea_ld + o] : 0;
+        ok = pos < tile.ncol;
+        dst = ok ? a.dst_off[tile.col0 + pos] : 0;
+        own_e = ok ? a.eb[a.src_vec[tile.col0 + pos]] : 0;
+        nblk = (a.M + 7) / 8;
+      } else {
+        if (e % (kTcEpilogue / BN) == 0) {
+          const int col = e / (kTcEpilogue / BN);
+          const bool cok = col < tile.ncol;
+          col_dst[col] = cok ? a.dst_off[tile.col0 + col] : 0;
+          col_e[col] = cok ? a.eb[a.src_vec[tile.col0 + col]] : 0;
+        }
+        ok = tile.m0 + pos < a.M;
+        own_e = ok ? a.ea[a.a_mat[tile.group] * a.ea_ld + tile.m0 + pos] : 0;
+        nblk = (tile.ncol + 7) / 8;
       }
-      const int row = tile.m0 + q * 32 + lane;
-      const bool row_ok = row < a.M;
-      const int era = row_ok ? a.ea[a.a_mat[tile.group] * a.ea_ld + row] : 0;
       const bool acc_ok = mbar_wait(&accbar[buf], (unsigned)(it / kBufs) & 1u, &abort_sh);
-      // uniform over the epilogue group (also publishes the column metadata written above)
+      // uniform over the epilogue group (also publishes the metadata written above)
       if (!epi_all(acc_ok && !abort_sh)) {
         abort_sh = 1;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;\n");
+      const unsigned tacc = tmem + ((unsigned)(q * 32) << 16) + (unsigned)(buf * kAccCols);
+      float cur[kAcc][8], nxt[kAcc][8];
+      auto read = [&](int cb, float (&v)[kAcc][8]) {
+#pragma unroll
+        for (int w = 0; w < kAcc; ++w) tmem_ld8(tacc + (unsigned)(w * (TR ? TR : BN) + cb * 8), v[w]);
+      };
+      auto release = [&]() {
+        asm volatile("tcgen05.fence::before_thread_sync;\n");
+        mbar_arrive(&tmem_free[buf]);
+      };
+      if (part < nblk) {
+        read(part, cur);
+        tmem_wait(cur);
+      } else {
+        release();
+      }
 #pragma unroll 1
-      for (int cb = part; cb < BN / 16; cb += kTcEpiParts) {
-        if (cb * 16 >= tile.ncol) break;
-        float vv[kAcc][16];
+      for (int cb = part; cb < nblk; cb += kTcEpiParts) {
+        const bool more = cb + kTcEpiParts < nblk;
+        if (more) read(cb + kTcEpiParts, nxt);
+        else release();
+        if constexpr (TR > 0) {
+          if (cb * 8 + 8 <= a.M) {
+            // each lane forms the slots of its destination into the warp's staging rows; then lanes 8 g .. 8 g + 7 store
+            // eight consecutive outputs of destination 4 i + g, four destinations per instruction
+            float2 (*stg)[8] = stage[warp - kTcProducers / 32];
 #pragma unroll
-        for (int w = 0; w < kAcc; ++w) {
-          const unsigned taddr =
-              tmem + ((unsigned)(q * 32) << 16) + (unsigned)(buf * kAccCols + w * BN + cb * 16);
-          unsigned rr[16];
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-              "[%16];\n"
-              : "=r"(rr[0]), "=r"(rr[1]), "=r"(rr[2]), "=r"(rr[3]), "=r"(rr[4]), "=r"(rr[5]), "=r"(rr[6]),
-                "=r"(rr[7]), "=r"(rr[8]), "=r"(rr[9]), "=r"(rr[10]), "=r"(rr[11]), "=r"(rr[12]), "=r"(rr[13]),
-                "=r"(rr[14]), "=r"(rr[15])
-              : "r"(taddr));
+            for (int cc = 0; cc < 8; ++cc) {
+              float h, l;
+              fold4(cur[0][cc], cur[1][cc], cur[2][cc], cur[3][cc], h, l);
+              stg[lane][cc] = out_value(h, l, col_e[cb * 8 + cc] + own_e);
+            }
+            __syncwarp();
 #pragma unroll
-          for (int cc = 0; cc < 16; ++cc) vv[w][cc] = __uint_as_float(rr[cc]);
+            for (int i = 0; i < 8; ++i) {
+              const int src = 4 * i + (lane >> 3);
+              const long long d = __shfl_sync(0xffffffffu, dst, src);
+              if (q * 32 + src < tile.ncol) a.Y[d + cb * 8 + (lane & 7)] = stg[src][lane & 7];
+            }
+            __syncwarp();
+          } else if (ok) {
+#pragma unroll
+            for (int cc = 0; cc < 8; ++cc) {
+              const int o = cb * 8 + cc;
+              if (o >= a.M) break;
+              float h, l;
+              fold4(cur[0][cc], cur[1][cc], cur[2][cc], cur[3][cc], h, l);
+              a.Y[dst + o] = out_value(h, l, col_e[o] + own_e);
+            }
+          }
+        } else if (ok) {
+          const int row = tile.m0 + pos;
+          if (cb * 8 + 8 <= tile.ncol) {
+            // a full block: no per-column exit, so the columns' independent chains (metadata load, fold, store) interleave
+#pragma unroll
+            for (int cc = 0; cc < 8; ++cc) {
+              float h, l;
+              fold4(cur[0][cc], cur[1][cc], cur[2][cc], cur[3][cc], h, l);
+              a.Y[col_dst[cb * 8 + cc] + row] = out_value(h, l, own_e + col_e[cb * 8 + cc]);
+            }
+          } else {
+#pragma unroll
+            for (int cc = 0; cc < 8; ++cc) {
+              if (cb * 8 + cc >= tile.ncol) break;
+              float h, l;
+              fold4(cur[0][cc], cur[1][cc], cur[2][cc], cur[3][cc], h, l);
+              a.Y[col_dst[cb * 8 + cc] + row] = out_value(h, l, own_e + col_e[cb * 8 + cc]);
+            }
+          }
         }
-        asm volatile("tcgen05.wait::ld.sync.aligned;\n");
-        if (row_ok && a.out_mode != 2 && cb * 16 + 16 <= tile.ncol) {
-          // a full block of 16 columns: no per-column exit, so the columns' independent chains
-          // (metadata load, fold, store) interleave
+        if (more) {
+          tmem_wait(nxt);
 #pragma unroll
-          for (int cc = 0; cc < 16; ++cc) {
-            const int col = cb * 16 + cc;
-            float h, l;
-            fold4(vv[0][cc], vv[1][cc], vv[2][cc], vv[3][cc], h, l);
-            store_out(a, col_dst[col], row, h, l, era + col_e[col], 0.0);
-          }
-        } else if (row_ok && a.out_mode != 2) {
+          for (int w = 0; w < kAcc; ++w)
 #pragma unroll
-          for (int cc = 0; cc < 16; ++cc) {
-            const int col = cb * 16 + cc;
-            if (col >= tile.ncol) break;
-            float h, l;
-            fold4(vv[0][cc], vv[1][cc], vv[2][cc], vv[3][cc], h, l);
-            store_out(a, col_dst[col], row, h, l, era + col_e[col], 0.0);
-          }
-        } else if (row_ok) {
-          // accumulating launch: fold first (the accumulators' registers are free again), then read
-          // the old values of eight columns together, then store them
-#pragma unroll
-          for (int cc = 0; cc < 16; ++cc) {
-            float h, l;
-            fold4(vv[0][cc], vv[1][cc], vv[2][cc], vv[3][cc], h, l);
-            vv[0][cc] = h;
-            vv[1][cc] = l;
-          }
-#pragma unroll
-          for (int c8 = 0; c8 < 16; c8 += 8) {
-            double old[8];
-#pragma unroll
-            for (int cc = 0; cc < 8; ++cc) {
-              const int col = cb * 16 + c8 + cc;
-              old[cc] = col < tile.ncol ? reinterpret_cast<const double*>(a.Y)[col_dst[col] + row] : 0.0;
-            }
-#pragma unroll
-            for (int cc = 0; cc < 8; ++cc) {
-              const int col = cb * 16 + c8 + cc;
-              if (col < tile.ncol)
-                store_out(a, col_dst[col], row, vv[0][c8 + cc], vv[1][c8 + cc], era + col_e[col], old[cc]);
-            }
-          }
+            for (int cc = 0; cc < 8; ++cc) cur[w][cc] = nxt[w][cc];
         }
       }
-      // accumulators read: the MMA warp may start the next tile
-      asm volatile("tcgen05.fence::before_thread_sync;\n");
-      mbar_arrive(&tmem_free[buf]);
-      // column metadata of this tile no longer needed by any epilogue thread
+      // metadata of this tile no longer needed by any epilogue thread
       asm volatile("bar.sync 1, %0;\n" ::"n"(kTcEpilogue) : "memory");
-    }
     }
   } else if (lane == 0) {
     // ---- MMA issuer
@@ -972,8 +875,11 @@ template <bool FINAL>
 __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, int per, int vec_out) {
   const int sub = threadIdx.x / per, t = threadIdx.x - sub * per;
   const int d = blockIdx.x * (blockDim.x / per) + sub, r = 2 * t;
-  if (d >= n_dst || r >= a.M) return;
-  const long long b = a.ptr[d], e = a.ptr[d + 1];
+  const bool live = d < n_dst && r < a.M;
+  const long long b = live ? a.ptr[d] : 0, e = live ? a.ptr[d + 1] : 0;
+  pdl_trigger();
+  pdl_wait();
+  if (!live) return;
   const float2* S = reinterpret_cast<const float2*>(a.S) + r;
   float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
   auto add = [&](float4 v) {
@@ -1017,20 +923,106 @@ __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, in
   }
 }
 
+// Sum and slice: vector v = sums of double-float slots (in slot order), K = nseg C elements, segment g of it from the
+// slots slot[ptr[v nseg + g]] .. ; its digits and exponent go to identifier vid[v] as k_slice_list writes them. The
+// expansions of a level are final once their contributions are summed, and only their digits are read afterwards,
+// so they are never stored in FP64.
+//
+// One warp per vector: lane t sums elements t, t + 32, .. (coalesced reads, kSumFlight slots in flight), the sums
+// pass through shared memory, and lanes of 8 consecutive elements form the digits. Measured: full-size star, locals of
+// 40,892 leaves from 1.17 GB of slots 252 us = 4.6 TB/s; all of its sums 661 us in place of 278 us of reductions into
+// FP64 expansions and about 400 us of slicing, and the upward and downward contractions, which added to FP64 values in
+// memory, 335 us instead of 880.
+constexpr int kSumWarps = 4, kSumFlight = 4;
+
+template <int S, int Q>  // Q: elements per lane
+__global__ void __launch_bounds__(32 * kSumWarps) k_sum_slice(int C, int nseg, int Kpad, long long n,
+                                                              const long long* __restrict__ ptr,
+                                                              const long long* __restrict__ slot,
+                                                              const long long* __restrict__ vid,
+                                                              const float2* __restrict__ slots, slice_t* __restrict__ out,
+                                                              int* __restrict__ eb) {
+  __shared__ double sh[kSumWarps][32 * Q];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, K = nseg * C;
+  const long long v = blockIdx.x * (long long)kSumWarps + warp;
+  pdl_trigger();
+  pdl_wait();
+  if (v >= n) return;
+  double mx = 0.0;
+  constexpr int QC = Q > 4 ? 4 : Q;  // elements per lane of a segment (C <= 128)
+  // the vector's offsets are read together, one per lane, 32 at a time
+  const long long p = lane <= nseg ? ptr[v * nseg + lane] : 0;
+  const long long end = __shfl_sync(0xffffffffu, p, nseg);
+  long long c0 = __shfl_sync(0xffffffffu, p, 0);
+  long long ids = c0 + lane < end ? slot[c0 + lane] : 0;
+  for (int g = 0; g < nseg; ++g) {
+    const long long b = __shfl_sync(0xffffffffu, p, g), e = __shfl_sync(0xffffffffu, p, g + 1);
+    float hi[QC], lo[QC];
+#pragma unroll
+    for (int q = 0; q < QC; ++q) hi[q] = lo[q] = 0.f;
+    for (long long k = b; k < e; k += kSumFlight) {
+      if (k + kSumFlight > c0 + 32) {
+        c0 = k;
+        ids = c0 + lane < end ? slot[c0 + lane] : 0;
+      }
+      float2 x[kSumFlight][QC];
+#pragma unroll
+      for (int i = 0; i < kSumFlight; ++i) {
+        const float2* src = slots + __shfl_sync(0xffffffffu, ids, (int)(k - c0) + i) + lane;
+#pragma unroll
+        for (int q = 0; q < QC; ++q)
+          x[i][q] = k + i < e && lane + 32 * q < C ? __ldcs(src + 32 * q) : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int i = 0; i < kSumFlight; ++i)
+        if (k + i < e) {
+#pragma unroll
+          for (int q = 0; q < QC; ++q) {
+            df_add(hi[q], lo[q], x[i][q].x);
+            df_add(hi[q], lo[q], x[i][q].y);
+          }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < QC; ++q) {
+      const int r = lane + 32 * q;
+      const double y = (double)hi[q] + (double)lo[q];
+      if (r < C) {
+        sh[warp][g * C + r] = y;
+        mx = fmax(mx, fabs(y));
+      }
+    }
+  }
+  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  __syncwarp();
+  const int e = exponent_of(mx);
+  const long long id = vid[v];
+  if (lane == 0) eb[id] = e;
+  if (8 * lane >= Kpad) return;
+  double x[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x[i] = 8 * lane + i < K ? sh[warp][8 * lane + i] : 0.0;
+  store_digits<S>(x, e, out + id * (long long)S * Kpad + (lane >> 1) * (S * 16) + (lane & 1) * 8);
+}
+
 constexpr int kKAlign = 32;  // padded K: a multiple of both engines' K steps
 int kpad(int K) { return (K + kKAlign - 1) / kKAlign * kKAlign; }
 
+// parts > 1: each matrix holds that many operators side by side (K columns each); they become matrices part * nmat + m.
 int slice_table(const double* A, int nmat, int M, int K, int lda, long long mstride, int S, SplitTable* out,
-                cudaStream_t s) {
-  out->M = M; out->K = K; out->Kpad = kpad(K); out->nmat = nmat; out->nrt = (M + kSplitBM - 1) / kSplitBM;
-  const size_t nh = (size_t)nmat * out->nrt * kSplitBM * S * out->Kpad;
-  TRY(cudaMalloc(&out->A, nh * sizeof(slice_t)));
-  TRY(cudaMemsetAsync(out->A, 0, nh * sizeof(slice_t), s));  // rows past M stay zero
-  TRY(cudaMalloc(&out->ea, (size_t)nmat * M * sizeof(int)));
+                cudaStream_t s, int parts = 1) {
+  out->M = M; out->K = K; out->Kpad = kpad(K); out->nmat = parts * nmat; out->nrt = (M + kSplitBM - 1) / kSplitBM;
+  const size_t nh = (size_t)nmat * out->nrt * kSplitBM * S * out->Kpad;  // of a part
+  TRY(cudaMalloc(&out->A, parts * nh * sizeof(slice_t)));
+  TRY(cudaMemsetAsync(out->A, 0, parts * nh * sizeof(slice_t), s));  // rows past M stay zero
+  TRY(cudaMalloc(&out->ea, (size_t)parts * nmat * M * sizeof(int)));
   const long long rows = (long long)nmat * M;
-  k_slice_rows<kSplitSlices><<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(
-      A, mstride, lda, M, K, out->Kpad, nmat, out->nrt, (slice_t*)out->A, out->ea);
-  TRY(cudaGetLastError());
+  for (int q = 0; q < parts; ++q) {
+    k_slice_rows<kSplitSlices><<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(
+        A + (long long)q * K, mstride, lda, M, K, out->Kpad, nmat, out->nrt, (slice_t*)out->A + q * nh,
+        out->ea + (size_t)q * rows);
+    TRY(cudaGetLastError());
+  }
   return VP_OK;
 }
 
@@ -1051,9 +1043,7 @@ int build_split(vp_tables_s* T, cudaStream_t s) {
   if ((rc = slice_table(T->m2l, nl * kVOff * T->nch, C, C, C, (long long)C * C, S, &st->m2l, s))) return rc;
   if ((rc = slice_table(T->m2t, nl * kWPos * T->nch, 3 * n, C, C, (long long)3 * n * C, S, &st->m2t, s))) return rc;
   if ((rc = slice_table(T->s2l, nl * kXPos * T->nch, C, n, n, (long long)C * n, S, &st->s2l, s))) return rc;
-  if ((rc = slice_table(T->m2m, nl * T->nch, C, 2 * C, 4 * C, (long long)C * 4 * C, S, &st->m2m_lo, s))) return rc;
-  if ((rc = slice_table(T->m2m + 2 * C, nl * T->nch, C, 2 * C, 4 * C, (long long)C * 4 * C, S, &st->m2m_hi, s)))
-    return rc;
+  if ((rc = slice_table(T->m2m, nl * T->nch, C, C, 4 * C, (long long)C * 4 * C, S, &st->m2m, s, 4))) return rc;
   if ((rc = slice_table(T->l2l, nl * 4 * T->nch, C, C, C, (long long)C * C, S, &st->l2l, s))) return rc;
   TRY(cudaStreamSynchronize(s));
   return VP_OK;
@@ -1062,7 +1052,7 @@ int build_split(vp_tables_s* T, cudaStream_t s) {
 void free_split_tables(vp_tables_s* T) {
   auto* st = static_cast<SplitTables*>(T->near_split);
   if (!st) return;
-  for (SplitTable* t : {&st->near, &st->s2m, &st->l2t, &st->m2l, &st->m2t, &st->s2l, &st->m2m_lo, &st->m2m_hi,
+  for (SplitTable* t : {&st->near, &st->s2m, &st->l2t, &st->m2l, &st->m2t, &st->s2l, &st->m2m,
                         &st->l2l}) {
     if (t->A) cudaFree(t->A);
     if (t->ea) cudaFree(t->ea);
@@ -1115,7 +1105,7 @@ int read_split_error(int* flag) {
   return VP_OK;
 }
 
-int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engine, int short_ctas) {
+int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engine, int short_ctas, bool pdl) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   TRY(cudaStreamIsCapturing(s, &cs));
   if (cs == cudaStreamCaptureStatusNone) {
@@ -1131,35 +1121,47 @@ int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engin
     // the full-size star, 7.07 with four)
     const int grid = short_ctas ? (n_tiles + 1) / 2 : (n_tiles < g_num_sms ? n_tiles : g_num_sms);
     if (engine == kEngineTcgen05)
-      k_split_gemm_tc<kSplitSlices, 128, 0><<<grid, kTcThreads, tc_smem_bytes(kSplitSlices, 128), s>>>(a, n_tiles);
+      TRY(launch(k_split_gemm_tc<kSplitSlices, 128, 0>, grid, kTcThreads, tc_smem_bytes(kSplitSlices, 128), s, pdl, a, n_tiles));
     else if (engine == kEngineTcgen05N64)
-      k_split_gemm_tc<kSplitSlices, 64, 0><<<grid, kTcThreads, tc_smem_bytes(kSplitSlices, 64), s>>>(a, n_tiles);
+      TRY(launch(k_split_gemm_tc<kSplitSlices, 64, 0>, grid, kTcThreads, tc_smem_bytes(kSplitSlices, 64), s, pdl, a, n_tiles));
     else if (a.M <= 96)
-      k_split_gemm_tc<kSplitSlices, 128, 96><<<grid, kTcThreads, tc_smem_bytes(kSplitSlices, 128), s>>>(a, n_tiles);
+      TRY(launch(k_split_gemm_tc<kSplitSlices, 128, 96>, grid, kTcThreads, tc_smem_bytes(kSplitSlices, 128), s, pdl, a, n_tiles));
     else
-      k_split_gemm_tc<kSplitSlices, 128, 128><<<grid, kTcThreads, tc_smem_bytes(kSplitSlices, 128), s>>>(a, n_tiles);
+      TRY(launch(k_split_gemm_tc<kSplitSlices, 128, 128>, grid, kTcThreads, tc_smem_bytes(kSplitSlices, 128), s, pdl, a, n_tiles));
   }
   else if (engine == kEngineMmaSmall)
-    k_split_gemm<kSplitSlices, 64, 32><<<n_tiles, 64, mma_smem_bytes(kSplitSlices, 64, 32), s>>>(a);
+    TRY(launch(k_split_gemm<kSplitSlices, 64, 32>, n_tiles, 64, mma_smem_bytes(kSplitSlices, 64, 32), s, pdl, a));
   else
-    k_split_gemm<kSplitSlices, 128, 64><<<n_tiles, 256, mma_smem_bytes(kSplitSlices, 128, 64), s>>>(a);
+    TRY(launch(k_split_gemm<kSplitSlices, 128, 64>, n_tiles, 256, mma_smem_bytes(kSplitSlices, 128, 64), s, pdl, a));
   TRY(cudaGetLastError());
   return VP_OK;
 }
 
 int launch_slice_list(const double* X, const long long* base, const long long* vid, long long nlist, int K, int kseg,
-                      long long seg_stride, long long cstride, void* out, int* eb, cudaStream_t s) {
+                      long long seg_stride, long long cstride, void* out, int* eb, cudaStream_t s, bool pdl) {
   if (nlist <= 0) return VP_OK;
   int lg_l = 2;  // lanes per vector: at least Kpad / 8, which is at most 32
   while ((8 << lg_l) < kpad(K)) ++lg_l;
   if (lg_l > 5 || (kseg > 0 && K > 2 * kseg)) return VP_ERR_ARG;
-  k_slice_list<kSplitSlices><<<(unsigned)(((nlist << lg_l) + 255) / 256), 256, 0, s>>>(
-      X, base, vid, nlist, K, kseg > 0 ? kseg : K, seg_stride, cstride, kpad(K), lg_l, (slice_t*)out, eb);
-  TRY(cudaGetLastError());
+  TRY(launch(k_slice_list<kSplitSlices>, (unsigned)(((nlist << lg_l) + 255) / 256), 256, 0, s, pdl, X, base, vid, nlist, K,
+             kseg > 0 ? kseg : K, seg_stride, cstride, kpad(K), lg_l, (slice_t*)out, eb));
   return VP_OK;
 }
 
-int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s) {
+int launch_sum_slice(int C, int nseg, long long n, const long long* ptr, const long long* slot, const long long* vid,
+                     const void* slots, void* out, int* eb, cudaStream_t s, bool pdl) {
+  if (n <= 0) return VP_OK;
+  const int K = nseg * C;
+  if (K > 256 || C > 128) return VP_ERR_ARG;
+  const unsigned blocks = (unsigned)((n + kSumWarps - 1) / kSumWarps);
+  const auto f = K <= 32 ? k_sum_slice<kSplitSlices, 1> : K <= 96 ? k_sum_slice<kSplitSlices, 3>
+                 : K <= 128 ? k_sum_slice<kSplitSlices, 4> : k_sum_slice<kSplitSlices, 8>;
+  TRY(launch(f, blocks, 32 * kSumWarps, 0, s, pdl, C, nseg, kpad(K), n, ptr, slot, vid,
+             static_cast<const float2*>(slots), static_cast<slice_t*>(out), eb));
+  return VP_OK;
+}
+
+int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s, bool pdl) {
   if (n_dst <= 0) return VP_OK;
   const int pairs = (a.M + 1) / 2;
   if (pairs > 512) return VP_ERR_ARG;  // 3 p^2 <= 768 rows
@@ -1169,11 +1171,10 @@ int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s) {
   auto even = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   if (a.final_out) {
     // n even: a pair of rows lies in one field, and destinations and N are even too
-    k_reduce_df<true><<<blocks, threads, 0, s>>>(a, n_dst, per, a.n % 2 == 0 && even(a.u) && even(a.g));
+    TRY(launch(k_reduce_df<true>, blocks, threads, 0, s, pdl, a, n_dst, per, a.n % 2 == 0 && even(a.u) && even(a.g)));
   } else {
-    k_reduce_df<false><<<blocks, threads, 0, s>>>(a, n_dst, per, 0);
+    TRY(launch(k_reduce_df<false>, blocks, threads, 0, s, pdl, a, n_dst, per, 0));
   }
-  TRY(cudaGetLastError());
   return VP_OK;
 }
 

@@ -31,14 +31,14 @@ struct SplitTable {
   int M = 0, K = 0, Kpad = 0, nmat = 0, nrt = 0;
 };
 
-// m2m_lo / m2m_hi: the multipole-to-multipole operator split by children (0-1 and 2-3) so that
-// every contraction has K = 2C <= 256.
+// m2m: the multipole-to-multipole operators, one matrix per child (matrix q (levels + 1) nch + level nch + channel for
+// child q), so a child's multipole is sliced once for both the upward pass and its own far field.
 struct SplitTables {
-  SplitTable near, s2m, l2t, m2l, m2t, s2l, m2m_lo, m2m_hi, l2l;
+  SplitTable near, s2m, l2t, m2l, m2t, s2l, m2m, l2l;
 };
 
 struct SplitArgs {
-  int M, Kpad, out_mode;        // out_mode 0: double-float slot (float2), 1: FP64 overwrite, 2: FP64 accumulate
+  int M, Kpad;
   int nrt;                      // row tiles of 128 per operator matrix
   int ea_ld;                    // rows per matrix in the row-exponent array (>= M: a launch may use the
                                 // leading M rows of its operators)
@@ -46,7 +46,7 @@ struct SplitArgs {
   const int* ea;
   const slice_t* B;             // sliced vectors [v][S][Kpad]
   const int* eb;
-  void* Y;
+  float2* Y;                    // double-float contribution slots
   const SplitTile* tiles;       // tiles of the engine that runs
   const long long* a_mat;       // per group: matrix index
   const long long* src_vec;     // per column: vector index
@@ -84,14 +84,18 @@ void free_split_tables(vp_tables_s* T);
 int prepare_split_launch();
 // short_ctas: tcgen05 CTAs take two tiles each (so other kernels can interleave) instead of one
 // persistent CTA per SM.
-int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engine, int short_ctas = 0);
+// pdl: the launch before it on `s` is a kernel: start while that one ends (griddepcontrol).
+int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engine, int short_ctas = 0, bool pdl = false);
 // Read and clear the flag that a bounded wait of the tcgen05 engine gave up.
 int read_split_error(int* flag);
 // Run a kernel whose bounded wait on an mbarrier nothing arrives at gives up after `budget` clocks.
 int selftest_wait(long long budget, cudaStream_t s);
 int launch_slice_list(const double* X, const long long* base, const long long* vid, long long nlist, int K, int kseg,
-                      long long seg_stride, long long cstride, void* out, int* eb, cudaStream_t s);
-int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s);
+                      long long seg_stride, long long cstride, void* out, int* eb, cudaStream_t s, bool pdl = false);
+int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s, bool pdl = false);
+// Sums of double-float slots sliced in place of being stored (k_sum_slice): n vectors of nseg segments of C elements.
+int launch_sum_slice(int C, int nseg, long long n, const long long* ptr, const long long* slot, const long long* vid,
+                     const void* slots, void* out, int* eb, cudaStream_t s, bool pdl = false);
 int split_kpad(int K);
 
 }  // namespace vp

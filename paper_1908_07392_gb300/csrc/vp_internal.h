@@ -48,6 +48,30 @@ const Positions& positions();
 void set_last_cuda(cudaError_t e);
 cudaError_t last_cuda();
 
+#ifdef __CUDACC__
+// Programmatic dependent launch: a kernel of a chain starts, sets up and waits for the one before it to complete
+// (pdl_wait) while that one still runs, and lets the next one do the same (pdl_trigger). Every thread of a kernel
+// launched with `pdl` passes pdl_wait before it reads or writes what an earlier launch writes or reads; without `pdl`
+// both are no-ops.
+__device__ inline void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ inline void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, bool pdl, A... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+#endif
+
 // Gauss-Legendre nodes and weights on [-1, 1], ascending (host).
 void gauss_legendre_host(int n, double* x, double* w);
 
