@@ -699,7 +699,8 @@ const double* table_ptr(const vp_tables_s* T, int t) {
 // Trees up to this many nodes launch their chain with programmatic dependent launch: CTAs that wait for the launch before
 // them keep near-field ones off their SMs, which costs more than the latency saved once the near field fills the chip.
 // Measured with / without: 64 leaves 93 / 111 us, 150,000 nodes 296 / 331 us, 10.5M nodes 7.02 / 6.78 ms; layers, whose
-// near part is small, 856 / 897 us (always on).
+// near part is small, 856 / 897 us (always on). Not under stream capture: in a graph of several trees the SMs that
+// waiting CTAs hold are another tree's (batch of four: 688 with, 641 us without).
 constexpr long long kPdlNodes = 300000;
 
 int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
@@ -1316,6 +1317,9 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
   double* bufs[BUF_COUNT] = {nullptr, tr->mp, tr->loc, tr->lslot, tr->uslot};
   const bool overlap = !ev && !step_ev && tr->side;
   int step_no = 0;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  TRY(cudaStreamIsCapturing(s0, &cap));
+  const bool chain_pdl = tr->pdl && cap == cudaStreamCaptureStatusNone;
   bool src_ready = false, near_started = false, joined = !overlap, after_kernel = false;
   if (overlap) {
     TRY(cudaEventRecord(tr->ev_fork, s0));
@@ -1339,7 +1343,7 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
     }
     const cudaStream_t s = (!overlap || near_step || st.stage == VP_STAGE_OUTPUT) ? s0 : tr->side;
     // a launch of the chain may start while the one before it ends, unless an event lies between them
-    const bool pdl = tr->pdl && after_kernel && s == tr->side;
+    const bool pdl = chain_pdl && after_kernel && s == tr->side;
     if (s == tr->side) after_kernel = overlap && st.kind != 2;
     if (st.kind == 2) {
       const long long elems = tr->mp_elems ? tr->mp_elems : (long long)tr->n_boxes * T->E;
