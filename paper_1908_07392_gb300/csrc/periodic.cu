@@ -179,10 +179,10 @@ struct Columns {
   static constexpr int threads = Shape<LOGN>::NT * groups * cols;
 };
 
-// CTAs per SM the compiler leaves registers for: 64 a thread where CTAs are large and throughput counts, 80
-// (no spills) where they are small and a thread's own speed does (512^2: 64.5 -> 58.4 us; at 1024^2 80
-// registers are slower, 189 against 172 us).
-constexpr int resident(int threads) { return (threads >= 256 ? 1024 : 768) / threads; }
+// CTAs per SM the compiler leaves registers for: 64 a thread where CTAs are large and throughput counts, 128
+// (no spills) where they are small and a thread's own speed does (512^2: 64, 80 and 128 registers 64.5, 58.4 and 56.3
+// us; at 1024^2 more than 64 are slower, 189 against 172 us).
+constexpr int resident(int threads) { return (threads >= 256 ? 1024 : 512) / threads; }
 
 enum { RED_OR, RED_MAX };
 
