@@ -369,11 +369,9 @@ struct DevSplit {
 // Sliced-vector families (split precision): 0 leaf values (K = n), 1 (box, channel) multipoles (K = C),
 // 2 locals of leaves (K = E), 3 (box, channel) locals of internal boxes (K = C).
 constexpr int kVecFamilies = 4;
-struct DevSlice {
-  int family, buf, K, kseg;
-  long long seg_stride, cstride, n;
-  const long long* base;  // null: contiguous, b = v * cstride
-  const long long* vid;   // null: identity
+struct DevSlice {  // n consecutive vectors of K elements of a buffer
+  int family, buf, K;
+  long long n;
 };
 
 enum Table { T_NEAR, T_S2M, T_L2T, T_M2M, T_L2L, T_M2L, T_M2T, T_S2L };
@@ -432,7 +430,6 @@ struct vp_tree_s {
   double* d_xi = nullptr;
   double *mp = nullptr, *loc = nullptr, *lslot = nullptr, *uslot = nullptr;
   long long n_lslot = 0, n_uslot = 0;
-  int lslot_stride = 0, uslot_stride = 0;  // slot strides of a layer program (even: 16-byte aligned slots)
   std::vector<void*> allocs;  // every device allocation owned by the tree
   std::vector<vp::DevGemm> gemms;
   std::vector<vp::DevReduce> reduces;
@@ -609,20 +606,13 @@ int upload_split(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
   return VP_OK;
 }
 
-// A slicing step (split precision): contiguous over a whole family, or a listed subset.
-int add_slice(vp_tree_s* tr, int family, int buf, int K, int kseg, long long seg_stride, long long cstride,
-              long long n, const std::vector<long long>* base, const std::vector<long long>* vid, cudaStream_t s) {
-  DevSlice d{family, buf, K, kseg, seg_stride, cstride, n, nullptr, nullptr};
-  int rc;
-  long long* p = nullptr;
-  if (base) { if ((rc = dev_upload(tr, *base, &p, s))) return rc; d.base = p; }
-  if (vid) { if ((rc = dev_upload(tr, *vid, &p, s))) return rc; d.vid = p; }
-  if (n <= 0) return VP_OK;
+// A slicing step (split precision).
+void add_slice(vp_tree_s* tr, int family, int buf, int K, long long n) {
+  if (n <= 0) return;
   const double by = (double)n * (8.0 * K + 2.0 * kSplitSlices * split_kpad(K) + 4.0);
   tr->steps.push_back({3, (int)tr->slice_ops.size(), tr->cur_stage, 0.0, by});
   tr->bytes[tr->cur_stage] += by;
-  tr->slice_ops.push_back(d);
-  return VP_OK;
+  tr->slice_ops.push_back({family, buf, K, n});
 }
 
 // A sum-and-slice step.
@@ -862,7 +852,7 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
     };
     tr->pdl = tr->N <= kPdlNodes;
     tr->cur_stage = VP_STAGE_UPWARD;
-    if ((rc = add_slice(tr, 0, BUF_F, n, n, 0, n, tr->n_leaves, nullptr, nullptr, s))) return rc;
+    add_slice(tr, 0, BUF_F, n, tr->n_leaves);
     if ((rc = upload_gemm(tr, s2m, s))) return rc;
     for (int l = P.max_level; l >= 2; --l) {
       if ((rc = upload_gemm(tr, up[l], s))) return rc;  // children of level l (none at the deepest)
@@ -1003,8 +993,6 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
   const int n = T->n, C = T->C, E = T->E, nch = T->nch;
   constexpr int NC = 2;                  // velocity components
   const int Cs = (C + 1) & ~1, Us = (n + 1) & ~1;
-  tr->lslot_stride = Cs;
-  tr->uslot_stride = Us;
   const auto& B = P.boxes;
   const long long NB = (long long)B.size();
   auto kact = [&](int l) { return l >= 0 && l <= T->levels && T->kactive[l]; };
@@ -1378,8 +1366,7 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
       if (rc) return rc;
     } else if (st.kind == 3) {
       const DevSlice& d = tr->slice_ops[st.index];
-      const int rc = launch_slice_list(bufs_c[d.buf], d.base, d.vid, d.n, d.K, d.kseg, d.seg_stride, d.cstride,
-                                       tr->sv[d.family], tr->se[d.family], s, pdl);
+      const int rc = launch_slice(bufs_c[d.buf], d.n, d.K, tr->sv[d.family], tr->se[d.family], s, pdl);
       if (rc) return rc;
       if (overlap && d.family == 0 && !near_started) {
         TRY(cudaEventRecord(tr->ev_src, s));
@@ -1394,10 +1381,10 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
     } else if (st.kind == 5) {
       const DevReduce& d = tr->reduces[st.index];
       DFReduceArgs a{};
-      a.M = d.args.M; a.n = d.args.n; a.final_out = d.args.final_out; a.N = d.args.N;
+      a.M = d.args.M; a.n = d.args.n; a.N = d.args.N;
       a.dst_off = d.args.dst_off; a.ptr = d.args.ptr; a.slot = d.args.slot;
       a.S = bufs_c[d.src];
-      if (a.final_out) { a.u = u; a.g = g; } else { a.Y = bufs[d.dst]; }
+      a.u = u; a.g = g;
       const int rc = launch_reduce_df(a, d.n_dst, s, pdl);
       if (rc) return rc;
     } else if (st.kind == 8) {

@@ -24,7 +24,7 @@
 // 2^-59 of the row's largest value, below the 2^-53 of each FP64 operation. Twiddles carry 62 bits.
 // The multiplier is applied in FP64.
 // Measured per solution: 4096^2 2.70 ms (15.0 ms with FP64 radix-4 rows, transposes and a separate spectral
-// pass), 2048^2 0.564 ms (3.6), 512^2 58 us (about 250). The error against long double is 0.2 to 0.9 of the
+// pass), 2048^2 0.564 ms (3.6), 512^2 56 us (about 250). The error against long double is 0.2 to 0.9 of the
 // FP64 form's in the 2-norm (32^2 .. 2048^2; white noise, few modes, point forces). What bounds it: 2048^2 runs
 // at 2 to 2.4 instructions per clock and SM of 4, the integer pipe half busy, the rest latency (about 330
 // instructions per point and transform); 155 bytes per point of DRAM traffic would take 0.1 ms.

@@ -142,24 +142,19 @@ __device__ inline void store_digits(const double (&x)[8], int e, slice_t* o) {
   for (int d = 0; d < S; ++d) *reinterpret_cast<uint4*>(o + d * 16) = make_uint4(w[d][0], w[d][1], w[d][2], w[d][3]);
 }
 
-// Slice a list of vectors. Vector v (v < nlist) has identifier id = vid ? vid[v] : v and elements
-// x_k = X[b + (k / kseg) * seg_stride + k % kseg], k < K <= 2 kseg, b = base ? base[v] : v * cstride;
-// output out[id][Kpad / 16][s][16] (the S slices of each K step of 16 are contiguous, so one
-// column of a K step is one 32 S-byte block for the GEMM engines' gathers) and eb[id].
+// Slice the vectors x_v = X[v K .. v K + K), v < nvec: output out[v][Kpad / 16][s][16] (the S slices of each K step of
+// 16 are contiguous, so one column of a K step is one 32 S-byte block for the GEMM engines' gathers) and eb[v].
 //
 // L lanes per vector (a power of two, L >= Kpad / 8), a lane taking 8 consecutive elements: they are read once and
 // kept for the digits, and a slice of them is one 16-byte store (2-byte stores, six per element, and a second
 // read of the vector took 571 us an evaluation of the full-size star, now 459).
 // Measured: the star's leaf sources (40,897 vectors of 256) 79 -> 52 us = 4.0 TB/s.
 template <int S>
-__global__ void __launch_bounds__(256) k_slice_list(const double* __restrict__ X, const long long* __restrict__ base,
-                                                    const long long* __restrict__ vid, long long nlist, int K, int kseg,
-                                                    long long seg_stride, long long cstride, int Kpad, int lg_l,
-                                                    slice_t* __restrict__ out, int* __restrict__ eb) {
+__global__ void __launch_bounds__(256) k_slice(const double* __restrict__ X, long long nvec, int K, int Kpad, int lg_l,
+                                               slice_t* __restrict__ out, int* __restrict__ eb) {
   const int L = 1 << lg_l, l = threadIdx.x & (L - 1);
   const long long v = (blockIdx.x * 256ll + threadIdx.x) >> lg_l;
-  const bool ok = v < nlist;
-  const long long b = !ok ? 0 : (base ? base[v] : v * cstride);
+  const bool ok = v < nvec;
   pdl_trigger();
   pdl_wait();
   double x[8];
@@ -167,15 +162,14 @@ __global__ void __launch_bounds__(256) k_slice_list(const double* __restrict__ X
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int k = 8 * l + i;
-    x[i] = ok && k < K ? X[b + k + (k >= kseg ? seg_stride - kseg : 0)] : 0.0;
+    x[i] = ok && k < K ? X[v * K + k] : 0.0;
     mx = fmax(mx, fabs(x[i]));
   }
   for (int o = L >> 1; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (!ok || 8 * l >= Kpad) return;
   const int e = exponent_of(mx);
-  const long long id = vid ? vid[v] : v;
-  if (l == 0) eb[id] = e;
-  store_digits<S>(x, e, out + id * (long long)S * Kpad + (l >> 1) * (S * 16) + (l & 1) * 8);
+  if (l == 0) eb[v] = e;
+  store_digits<S>(x, e, out + v * (long long)S * Kpad + (l >> 1) * (S * 16) + (l & 1) * 8);
 }
 
 __device__ inline void df_add(float& hi, float& lo, float x) {
@@ -865,13 +859,13 @@ size_t tc_smem_bytes(int S, int BN) { return (size_t)kTcStages * S * (kTcA + BN 
 
 // ------------------------------------------------------------------ reduction
 
-// Reduction of double-float slots: y[dst] = sum of its slots (double-float, in slot order), written as FP64. A thread
+// The outputs from double-float slots: u and its gradient at a destination's points = the sum of its slots (double-float,
+// in slot order), written as FP64. A thread
 // sums two neighbouring rows (16-byte reads: slots start at even offsets), `per` threads a destination, as many
 // destinations to a block as fit; slot offsets come through L1 by broadcast, so a block waits for no barrier (one
 // destination per block of 256 threads, offsets staged in shared memory, left short destinations waiting on
 // latency: the coupled-step layer's output, 1 to 2 slots of 256 rows, 133 -> 51 us; long ones stream slots at the copy
 // rate either way, the full-size star's output 559 -> 580 us. More loads in flight cost occupancy: 6 took 782 us).
-template <bool FINAL>
 __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, int per, int vec_out) {
   const int sub = threadIdx.x / per, t = threadIdx.x - sub * per;
   const int d = blockIdx.x * (blockDim.x / per) + sub, r = 2 * t;
@@ -902,29 +896,20 @@ __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, in
     if (k + 2 < e) add(v2);
   }
   const double y0 = (double)h0 + (double)l0, y1 = (double)h1 + (double)l1;
-  double* y;
-  if (FINAL) {
-    const int f = r / a.n;
-    y = (f == 0 ? a.u : a.g + (f - 1) * a.N) + a.dst_off[d] + (r - f * a.n);
-    if (!vec_out && r + 1 < a.M) {  // the next row may begin another field
-      const int f1 = (r + 1) / a.n;
-      (f1 == 0 ? a.u : a.g + (f1 - 1) * a.N)[a.dst_off[d] + (r + 1 - f1 * a.n)] = y1;
-      *y = y0;
-      return;
-    }
-  } else {
-    y = a.Y + a.dst_off[d] + r;
-  }
+  auto out = [&](int row) {
+    const int f = row / a.n;
+    return (f == 0 ? a.u : a.g + (f - 1) * a.N) + a.dst_off[d] + (row - f * a.n);
+  };
   if (vec_out) {
-    *reinterpret_cast<double2*>(y) = make_double2(y0, y1);
+    *reinterpret_cast<double2*>(out(r)) = make_double2(y0, y1);
   } else {
-    y[0] = y0;
-    if (!FINAL && r + 1 < a.M) y[1] = y1;
+    *out(r) = y0;
+    if (r + 1 < a.M) *out(r + 1) = y1;  // may begin the next field
   }
 }
 
 // Sum and slice: vector v = sums of double-float slots (in slot order), K = nseg C elements, segment g of it from the
-// slots slot[ptr[v nseg + g]] .. ; its digits and exponent go to identifier vid[v] as k_slice_list writes them. The
+// slots slot[ptr[v nseg + g]] .. ; its digits and exponent go to identifier vid[v] as k_slice writes them. The
 // expansions of a level are final once their contributions are summed, and only their digits are read afterwards,
 // so they are never stored in FP64.
 //
@@ -1137,14 +1122,13 @@ int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engin
   return VP_OK;
 }
 
-int launch_slice_list(const double* X, const long long* base, const long long* vid, long long nlist, int K, int kseg,
-                      long long seg_stride, long long cstride, void* out, int* eb, cudaStream_t s, bool pdl) {
-  if (nlist <= 0) return VP_OK;
+int launch_slice(const double* X, long long nvec, int K, void* out, int* eb, cudaStream_t s, bool pdl) {
+  if (nvec <= 0) return VP_OK;
   int lg_l = 2;  // lanes per vector: at least Kpad / 8, which is at most 32
   while ((8 << lg_l) < kpad(K)) ++lg_l;
-  if (lg_l > 5 || (kseg > 0 && K > 2 * kseg)) return VP_ERR_ARG;
-  TRY(launch(k_slice_list<kSplitSlices>, (unsigned)(((nlist << lg_l) + 255) / 256), 256, 0, s, pdl, X, base, vid, nlist, K,
-             kseg > 0 ? kseg : K, seg_stride, cstride, kpad(K), lg_l, (slice_t*)out, eb));
+  if (lg_l > 5) return VP_ERR_ARG;
+  TRY(launch(k_slice<kSplitSlices>, (unsigned)(((nvec << lg_l) + 255) / 256), 256, 0, s, pdl, X, nvec, K, kpad(K), lg_l,
+             (slice_t*)out, eb));
   return VP_OK;
 }
 
@@ -1169,12 +1153,8 @@ int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s, bool pdl)
   const int per = (pairs + 31) / 32 * 32, threads = per >= 96 ? per : 128 / per * per;
   const unsigned blocks = (unsigned)((n_dst + threads / per - 1) / (threads / per));
   auto even = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  if (a.final_out) {
-    // n even: a pair of rows lies in one field, and destinations and N are even too
-    TRY(launch(k_reduce_df<true>, blocks, threads, 0, s, pdl, a, n_dst, per, a.n % 2 == 0 && even(a.u) && even(a.g)));
-  } else {
-    TRY(launch(k_reduce_df<false>, blocks, threads, 0, s, pdl, a, n_dst, per, 0));
-  }
+  // n even: a pair of rows lies in one field, and destinations and N are even too
+  TRY(launch(k_reduce_df, blocks, threads, 0, s, pdl, a, n_dst, per, a.n % 2 == 0 && even(a.u) && even(a.g)));
   return VP_OK;
 }
 

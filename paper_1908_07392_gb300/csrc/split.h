@@ -54,13 +54,12 @@ struct SplitArgs {
 };
 
 struct DFReduceArgs {
-  int M, n, final_out;
+  int M, n;
   long long N;
   const long long* dst_off;
   const long long* ptr;
   const long long* slot;
   const void* S;
-  double* Y;
   double* u;
   double* g;
 };
@@ -90,8 +89,8 @@ int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engin
 int read_split_error(int* flag);
 // Run a kernel whose bounded wait on an mbarrier nothing arrives at gives up after `budget` clocks.
 int selftest_wait(long long budget, cudaStream_t s);
-int launch_slice_list(const double* X, const long long* base, const long long* vid, long long nlist, int K, int kseg,
-                      long long seg_stride, long long cstride, void* out, int* eb, cudaStream_t s, bool pdl = false);
+// nvec consecutive vectors of K elements into digits and exponents (k_slice).
+int launch_slice(const double* X, long long nvec, int K, void* out, int* eb, cudaStream_t s, bool pdl = false);
 int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s, bool pdl = false);
 // Sums of double-float slots sliced in place of being stored (k_sum_slice): n vectors of nseg segments of C elements.
 int launch_sum_slice(int C, int nseg, long long n, const long long* ptr, const long long* slot, const long long* vid,
