@@ -46,11 +46,11 @@ FP64_FLOPS_PER_CLK_PER_SM = 4.0   # 2 DFMA per clock per SM: 1.25 TFLOP/s nomina
 TRAFFIC_FP64_NEAR = 3.68e9
 TRAFFIC_FP64_NEAR_SOURCE = "constant from a past ncu capture (profiles/near_f64_star_d8.md, depth 8 scaled by near pairs)"
 # DRAM bytes of the split-precision near-field launch (tcgen05 engine) per algorithmic GFLOP of the near
-# stage, NOT measured in this run: the ncu capture of the same kernel at depth 8 (419.3 MB read + 419.2
+# stage, NOT measured in this run: the ncu capture of the same kernel at depth 8 (491.8 MB read + 425.5
 # MB written for 29.33 GFLOP, profiles/near_tc_star_d8.md); traffic grows with the near pairs, i.e. with
 # the stage's flops.
-TRAFFIC_SPLIT_NEAR_PER_GFLOP = 838.5e6 / 29.33
-TRAFFIC_SPLIT_NEAR_SOURCE = ("constant from an ncu capture (profiles/near_tc_star_d8.md, depth 8, 838.5 MB for 29.33 "
+TRAFFIC_SPLIT_NEAR_PER_GFLOP = 917.3e6 / 29.33
+TRAFFIC_SPLIT_NEAR_SOURCE = ("constant from an ncu capture (profiles/near_tc_star_d8.md, depth 8, 917.3 MB for 29.33 "
                              "GFLOP) scaled by the near stage's flops")
 N_SM = 152
 ENGINE_NAMES = {-1: "-", 0: "mma.sync 128x64", 1: "tcgen05 128x128", 2: "mma.sync 64x32", 3: "tcgen05 128x64",
@@ -475,16 +475,17 @@ def periodic_and_sdc(args, V, steps, warmup, flush, stream):
     finally:
         P.close()
     med = statistics.median(ms)
-    flops = 4 * 10.0 * n * n * np.log2(n)  # one forward and three inverse complex 2-D transforms (nominal count)
-    fp64_peak = N_SM * 2070.0e6 * FP64_FLOPS_PER_CLK_PER_SM / 1e12
+    nbytes = 64.0 * n * n  # the force read once, the velocity and its gradient written once
+    hbm = measured_peaks().get("hbm_gbs", 6800.0)
     out["periodic_fft"] = {
         "workload": f"periodic modified Stokes velocity and gradient on a {n}^2 grid, box side 3, alpha 316",
         "value": n * n / (med / 1e3), "unit": "grid points/s", "ms_per_eval": med, "steps": steps,
         "rel_err_vs_manufactured": err,
-        "roofline": {"bound": "alu", "kernel": "k_fft_rows: FP64 radix-4 Stockham rows in shared memory",
-                     "achieved": flops / (med / 1e3) / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
-                     "frac": flops / (med / 1e3) / 1e12 / fp64_peak,
-                     "flops_note": "10 n^2 log2 n per complex 2-D transform, 4 transforms"}}
+        "roofline": {"bound": "hbm", "kernel": "k_rows_forward, k_columns, k_rows_inverse: radix-8 Stockham on 64-bit "
+                                               "integers in shared memory",
+                     "achieved": nbytes / (med / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
+                     "frac": nbytes / (med / 1e3) / 1e9 / hbm, "peak_source": "measured copy, of measured",
+                     "note": "algorithmic bytes; issue of the integer instructions and latency bound it, not memory"}}
     # SISDC time stepping on the periodic box: Taylor-Green vortex, exact decay exp(-2 t / Re)
     n, re, dt = 2048, 1.0, 0.01
     u0, g0, l0 = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in I.taylor_green(n))
@@ -639,7 +640,7 @@ def run_steps(args):
             "plain_mean_iters": r["plain_mean_iters"], "volume_ms_mean": r["volume_ms_mean"],
             "train_seconds": r["train_seconds"], "train_loss": [r["first_train_loss"], r["final_train_loss"]],
             "interior_rel_err_exact_solution": err, "wall_seconds": wall,
-            "gmres_operator_roofline": {"kernel": "k_gemv (dense FP64 Nystrom matrix)", "bound": "hbm",
+            "gmres_operator_roofline": {"kernel": "k_gemv (dense Nystrom matrix, 63-bit integers)", "bound": "hbm",
                                         "achieved": gemv_bytes / (gemv_ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                                         "frac": gemv_bytes / (gemv_ms / 1e3) / 1e9 / hbm, "ms": gemv_ms},
             "clocks": sampler.summary()}

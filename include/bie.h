@@ -24,7 +24,8 @@ extern "C" {
 typedef struct bie_s* bie;
 
 /*
- * bie_create -- nodes and the dense FP64 Nystrom matrix (2N x 2N, on the device) for alpha > 0.
+ * bie_create -- nodes and the dense Nystrom matrix (2N x 2N, on the device) for alpha > 0: computed in FP64 and kept as
+ * 63-bit integers with one exponent per row (rounding 2^-63 of a row's largest entry), the diagonal apart in FP64.
  * Entries from the target's own panel and its two neighbours come from a graded local quadrature
  * of the kernel against the panel's Lagrange basis (the kernel's r log r terms); the rest are plain
  * Gauss-Legendre. max_krylov (1..1000) sizes the GMRES work space. Synchronises `stream`.

@@ -308,7 +308,7 @@ void vp_layer_free(vp_layer layer);
  * alpha^2) and its gradient by Fourier differentiation (the Nyquist mode differentiates to zero).
  * The paper feeds it the PUX extension of the force; here the caller supplies a periodic force.
  * vp_periodic_create -- plan for alpha > 0, n a power of two in 32..4096, side L > 0 (work arrays of
- *  4 n^2 complex doubles on the device; synchronises `stream`).
+ *  3 n^2 16-byte complex integers and (n/2 + 1)^2 doubles on the device; synchronises `stream`).
  * vp_periodic_eval -- F device [2][n][n] (component, row j, column i), u device [2][n][n], gradu
  *  device [2][2][n][n] with gradu[a][m] = d u_a / d x_m. Calls on one plan must not overlap.
  * Errors: VP_ERR_ARG, VP_ERR_OOM, VP_ERR_CUDA.
@@ -386,7 +386,8 @@ int vp_eval_static(vp_tree tree, const double* f, double* u, double* gradu, void
  *  4  tcgen05 on transposed tiles: the tile's 128 columns are the MMA's rows and the operator's rows
  *     its N (rounded up to 96 or 128), so operators of at most 128 rows (the 81-row multipole and
  *     local operators) fill every tensor-memory lane; launches with taller operators run on engine 1.
- * All compute the same exact slice sums. vp_tree_set_engine sets one engine for every launch of
+ * All compute the same exact slice sums. Until a tree is tuned its launches use engines 1, 3 and 4, by rows and number
+ * of tiles. vp_tree_set_engine sets one engine for every launch of
  * the tree (VP_ERR_ARG for other values). vp_autotune times each split-precision launch of one
  * evaluation of `f` with every engine (tile shape) on `stream`, keeps the fastest per launch shape,
  * evaluates once more into u, gradu with the choice, and, if *n_tcgen05 is given, reports how many

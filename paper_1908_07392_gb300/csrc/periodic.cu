@@ -27,7 +27,8 @@
 // pass), 2048^2 0.564 ms (3.6), 512^2 56 us (about 250). The error against long double is 0.2 to 0.9 of the
 // FP64 form's in the 2-norm (32^2 .. 2048^2; white noise, few modes, point forces). What bounds it: 2048^2 runs
 // at 2 to 2.4 instructions per clock and SM of 4, the integer pipe half busy, the rest latency (about 330
-// instructions per point and transform); 155 bytes per point of DRAM traffic would take 0.1 ms.
+// instructions per point and transform), 4096^2 at 1.4 with one CTA of k_columns per SM (registers); 155 bytes per
+// point of DRAM traffic would take 0.1 ms.
 #include <cuda_runtime.h>
 
 #include <cmath>

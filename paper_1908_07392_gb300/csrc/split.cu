@@ -403,11 +403,8 @@ size_t mma_smem_bytes(int S, int BM, int BN) { return (size_t)2 * S * (BM + BN) 
 __device__ int g_split_error = 0;
 
 constexpr int kTcProducers = 96;                  // warps 0-2
-#ifndef VP_TC_EPILOGUE_WARPS
-#define VP_TC_EPILOGUE_WARPS 16
-#endif
-constexpr int kTcEpilogue = 32 * VP_TC_EPILOGUE_WARPS;  // warps 3 .. 18
-constexpr int kTcEpiParts = VP_TC_EPILOGUE_WARPS / 4;   // epilogue warps per tensor-memory lane quadrant
+constexpr int kTcEpilogue = 512;                  // warps 3 .. 18
+constexpr int kTcEpiParts = kTcEpilogue / 128;    // epilogue warps per tensor-memory lane quadrant
 constexpr int kTcMmaWarp = (kTcProducers + kTcEpilogue) / 32;
 constexpr int kTcThreads = kTcProducers + kTcEpilogue + 32;
 constexpr int kTcKC = 16;                         // K per stage
