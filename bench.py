@@ -41,9 +41,9 @@ sys.path.insert(0, ROOT)
 
 FP64_FLOPS_PER_CLK_PER_SM = 4.0   # 2 DFMA per clock per SM: 1.25 TFLOP/s nominal over 152 SMs at ~2.06 GHz
 # DRAM bytes of one FP64 near-field launch on the default workload, NOT measured in this run: a past ncu
-# capture of the same kernel at depth 8 (688 MB for 66.6k near pairs, profiles/near_f64_star_d8.md) scaled
+# capture of the same kernel at depth 8 (692 MB for 66.6k near pairs, profiles/near_f64_star_d8.md) scaled
 # by pairs to the 356k pairs at depth 10.
-TRAFFIC_FP64_NEAR = 3.68e9
+TRAFFIC_FP64_NEAR = 3.70e9
 TRAFFIC_FP64_NEAR_SOURCE = "constant from a past ncu capture (profiles/near_f64_star_d8.md, depth 8 scaled by near pairs)"
 # DRAM bytes of the split-precision near-field launch (tcgen05 engine) per algorithmic GFLOP of the near
 # stage, NOT measured in this run: the ncu capture of the same kernel at depth 8 (491.8 MB read + 425.5
