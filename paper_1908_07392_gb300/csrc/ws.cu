@@ -219,12 +219,13 @@ int launch_conv_k(int n, int B, int Cin, int Cout, const float* W, const float* 
 // the allocation on.
 __global__ void k_layout(int Cin, int Cout, int K, const float* __restrict__ p, float* __restrict__ wf,
                          float* __restrict__ wb) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= Cin * Cout * K) return;
-  const int o = e / (Cin * K), rem = e - o * Cin * K, c = rem / K, k = rem - c * K;
+  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;  // layers of 2^31 weights and more are accepted
+  if (e >= (size_t)Cin * Cout * K) return;
+  const int c = (int)(e / K % Cin), k = (int)(e % K);
+  const size_t o = e / K / Cin;
   const float v = p[e];
-  wf[(size_t)(c * K + k) * pad4(Cout) + o] = v;
-  wb[(size_t)(o * K + K - 1 - k) * pad4(Cin) + c] = v;
+  wf[((size_t)c * K + k) * pad4(Cout) + o] = v;
+  wb[(o * K + K - 1 - k) * pad4(Cin) + c] = v;
 }
 
 // Part sums of dW[o][c][k] = sum_{b,x} dz[b][o][x] a[b][c][(x + k - K/2) mod n] and dbias[o] = sum dz over a
@@ -391,9 +392,10 @@ int wgrad_segs(size_t layer_params) {
 
 // g[p] = sum over the segments of part[seg][p], compensated: 32 parameters per block, warp w taking the
 // segments w mod 8, the eight sums added in their order.
-__global__ void __launch_bounds__(256) k_sum_parts(int m, int segs, const float* __restrict__ part, float* __restrict__ g) {
+__global__ void __launch_bounds__(256) k_sum_parts(size_t m, int segs, const float* __restrict__ part, float* __restrict__ g) {
   __shared__ float2 sh[8][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t p = blockIdx.x * (size_t)32 + lane;
   float s = 0.f, e = 0.f;
   auto add = [&](float v) {
     const float t = s + v, bb = t - s;
@@ -402,7 +404,7 @@ __global__ void __launch_bounds__(256) k_sum_parts(int m, int segs, const float*
   };
   if (p < m) {
 #pragma unroll 8
-    for (int q = w; q < segs; q += 8) add(part[(size_t)q * m + p]);
+    for (int q = w; q < segs; q += 8) add(part[q * m + p]);
   }
   sh[w][lane] = make_float2(s, e);
   __syncthreads();
@@ -525,7 +527,7 @@ int grad(ws_s* w, const float* x, const float* t, int B, float* loss, cudaStream
     const size_t m = (size_t)Cout * Cin * w->K + Cout;  // weights, then bias
     const int segs = wgrad_segs(m);
     if ((rc = wgrad_of(w->K)(w->n, B, Cin, Cout, dz, a, w->wparts, segs, s))) return rc;
-    k_sum_parts<<<(unsigned)((m + 31) / 32), 256, 0, s>>>((int)m, segs, w->wparts, w->g + w->woff[l]);
+    k_sum_parts<<<(unsigned)((m + 31) / 32), 256, 0, s>>>(m, segs, w->wparts, w->g + w->woff[l]);
     TRY(cudaGetLastError());
     if (l > 0) {
       // da masked by the activation of the layer
