@@ -12,7 +12,7 @@ LIB = os.path.join(BUILD, "libvp.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["tables.cu", "eval.cu", "split.cu", "bie.cu", "ws.cu", "layer.cu", "periodic.cu", "sdc.cu"]
 CPP_SOURCES = ["plan.cpp"]
-HEADERS = ["special.cuh", "stokes.cuh", "layer.h", "vp_internal.h", "plan.h", "split.h", os.path.join("..", "..", "include", "vp.h"),
+HEADERS = ["special.cuh", "stokes.cuh", "layer.h", "vp_internal.h", "plan.h", "split.h", "fsum.h", os.path.join("..", "..", "include", "vp.h"),
            os.path.join("..", "..", "include", "bie.h")]
 
 

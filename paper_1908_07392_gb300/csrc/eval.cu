@@ -396,7 +396,7 @@ struct HostSum {
 struct DevPt {
   PtInst* inst = nullptr;
   int n_inst = 0, rows = 0, rb = 0, dst = 0;
-  long long bs = 0;
+  long long bs = 0, rem = 0;  // rem: offset of the slots of remainders (launch_pt_apply)
   double* A = nullptr;
 };
 
@@ -959,7 +959,7 @@ struct LayerBins {
 };
 
 int upload_pt(vp_tree_s* tr, std::vector<PtInst>& inst, int rows, int rb, long long bs, int dst_buf, int kind,
-              const PtSources& S, cudaStream_t s) {
+              const PtSources& S, cudaStream_t s, long long rem = 0) {
   if (inst.empty()) return VP_OK;
   const vp_tables_s* T = tr->T;
   long long total = 0;
@@ -972,7 +972,7 @@ int upload_pt(vp_tree_s* tr, std::vector<PtInst>& inst, int rows, int rb, long l
     fl += 2.0 * rows * 2.0 * I.ns;
   }
   DevPt d;
-  d.n_inst = (int)inst.size(); d.rows = rows; d.rb = rb; d.bs = bs; d.dst = dst_buf;
+  d.n_inst = (int)inst.size(); d.rows = rows; d.rb = rb; d.bs = bs; d.rem = rem; d.dst = dst_buf;
   int rc;
   if ((rc = dev_upload(tr, inst, &d.inst, s))) return rc;
   void* A = nullptr;
@@ -1025,8 +1025,12 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
     I.j0 = bins.first[i]; I.ns = bins.count[i]; I.kact = kact(b.level); I.dst = split ? nup : off(0, i);
     ps2m.push_back(I);
     if (!split) continue;
-    for (int a = 0; a < NC; ++a, nup += Es)
-      for (int ch = 0; ch < nch; ++ch) upl[(size_t)(a * NB + i) * nch + ch].push_back(nup + ch * C);
+    // a slot per component, then those of the remainders: the sources' FP64 sums enter whole
+    for (int a = 0; a < NC; ++a)
+      for (int ch = 0; ch < nch; ++ch)
+        for (int part = 0; part < 2; ++part)
+          upl[(size_t)(a * NB + i) * nch + ch].push_back(nup + (part * NC + a) * Es + ch * C);
+    nup += 2 * NC * Es;
   }
   HostGemm m2l, l2t, m2t;
   m2l.M = C; m2l.K = C; m2l.lda = C; m2l.table = T_M2L; m2l.src = BUF_MP; m2l.dst = BUF_LSLOT; m2l.split_vec = 1;
@@ -1168,7 +1172,7 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
     };
     tr->pdl = true;
     tr->cur_stage = VP_STAGE_UPWARD;
-    if ((rc = upload_pt(tr, ps2m, 2 * E, E, Es, BUF_MP, 0, S, s))) return rc;
+    if ((rc = upload_pt(tr, ps2m, 2 * E, E, Es, BUF_MP, 0, S, s, NC * Es))) return rc;
     for (int l = P.max_level; l >= 2; --l) {
       if ((rc = upload_gemm(tr, up[l], s))) return rc;
       if ((rc = add_sum(l, true))) return rc;
@@ -1363,7 +1367,7 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
       const DevPt& d = tr->pts[st.index];
       // slots of split-precision trees hold double-float values
       const int df = T->precision == VP_PREC_SPLIT;
-      const int rc = launch_pt_apply(d.rows, d.rb, d.bs, df, d.inst, d.n_inst, tr->d_perm, bufs_c[BUF_F], d.A,
+      const int rc = launch_pt_apply(d.rows, d.rb, d.bs, df, d.rem, d.inst, d.n_inst, tr->d_perm, bufs_c[BUF_F], d.A,
                                      bufs[d.dst], s);
       if (rc) return rc;
     } else if (st.kind == 3) {

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(256) k_pt_near(double alpha, int p, const doub
 constexpr int kApplyThreads = 256, kApplyRows = 4, kApplyChunk = 1024;
 
 __global__ void __launch_bounds__(kApplyThreads) k_pt_apply(int rows, int rb, long long bs, int df,
-                                                             const PtInst* inst, const int* perm, const double* mu,
+                                                             long long rem, const PtInst* inst, const int* perm, const double* mu,
                                                              const double* A, double* Y) {
   __shared__ double xs[kApplyChunk];
   const PtInst I = inst[blockIdx.x];
@@ -163,8 +163,9 @@ __global__ void __launch_bounds__(kApplyThreads) k_pt_apply(int rows, int rb, lo
     const long long o = I.dst + (long long)(r / rb) * bs + r % rb;
     if (df) {
       // double-float slot (the contribution slots of split-precision trees): high and low fp32 parts
-      const float h = __double2float_rn(acc[q]);
-      reinterpret_cast<float2*>(Y)[o] = make_float2(h, __double2float_rn(acc[q] - (double)h));
+      const float h = __double2float_rn(acc[q]), l = __double2float_rn(acc[q] - (double)h);
+      reinterpret_cast<float2*>(Y)[o] = make_float2(h, l);
+      if (rem) reinterpret_cast<float2*>(Y)[o + rem] = make_float2(__double2float_rn((acc[q] - (double)h) - (double)l), 0.f);
     } else {
       Y[o] = acc[q];
     }
@@ -192,11 +193,11 @@ int launch_pt_near(double alpha, int p, const double* xi, const PtInst* inst, in
   return VP_OK;
 }
 
-int launch_pt_apply(int rows, int rb, long long bs, int df, const PtInst* inst, int n_inst, const int* perm,
-                    const double* mu, const double* A, double* Y, cudaStream_t s) {
+int launch_pt_apply(int rows, int rb, long long bs, int df, long long rem, const PtInst* inst, int n_inst,
+                    const int* perm, const double* mu, const double* A, double* Y, cudaStream_t s) {
   if (n_inst <= 0) return VP_OK;
   if (rows > kApplyThreads * kApplyRows || rb <= 0) return VP_ERR_ARG;
-  k_pt_apply<<<(unsigned)n_inst, kApplyThreads, 0, s>>>(rows, rb, bs, df, inst, perm, mu, A, Y);
+  k_pt_apply<<<(unsigned)n_inst, kApplyThreads, 0, s>>>(rows, rb, bs, df, rem, inst, perm, mu, A, Y);
   TRY(cudaGetLastError());
   return VP_OK;
 }

@@ -36,9 +36,10 @@ int launch_pt_near(double alpha, int p, const double* xi, const PtInst* inst, in
                    PtSources src, double* A, cudaStream_t s);
 // Y[dst + (row / rb) bs + row % rb] = sum over columns of A times the density (mu interleaved
 // (mu_x, mu_y) per source), one block per instance; df != 0 writes double-float (two fp32) values,
-// the slot format of split-precision trees, into the 8-byte elements of Y.
-int launch_pt_apply(int rows, int rb, long long bs, int df, const PtInst* inst, int n_inst, const int* perm,
-                    const double* mu, const double* A, double* Y, cudaStream_t s);
+// the slot format of split-precision trees, into the 8-byte elements of Y, and with rem != 0 what those leave of the
+// FP64 value into the element `rem` further on, a slot of its own.
+int launch_pt_apply(int rows, int rb, long long bs, int df, long long rem, const PtInst* inst, int n_inst,
+                    const int* perm, const double* mu, const double* A, double* Y, cudaStream_t s);
 
 }  // namespace vp
 

@@ -27,6 +27,7 @@
 #include <new>
 #include <vector>
 
+#include "fsum.h"
 #include "plan.h"
 #include "split.h"
 #include "vp_internal.h"
@@ -102,31 +103,17 @@ __global__ void k_slice_rows(const double* __restrict__ A, long long mstride, in
   if (lane == 0) ea[mat * M + r] = e;
 }
 
-// The S digits (digits()) of 8 consecutive elements with the vector's exponent e, one 16-byte store per slice. With 128
-// added to each of the lower five, balanced digits are plain bytes, and a byte under the bits of 2^23 is a float
-// that one multiply-add turns into (byte - 128) 2^(-8 (i + 1)), exact.
+// The S digits (digits()) of 8 consecutive elements from T = round(|x| 2^(8S - e)) and the signs (bit i of `neg`), one
+// 16-byte store per slice. With 128 added to each of the lower five, balanced digits are plain bytes, and a byte under
+// the bits of 2^23 is a float that one multiply-add turns into (byte - 128) 2^(-8 (i + 1)), exact.
 template <int S>
-__device__ inline void store_digits(const double (&x)[8], int e, slice_t* o) {
+__device__ inline void store_digits(const unsigned long long (&t)[8], unsigned neg, slice_t* o) {
   static_assert(S == 6, "five balanced bytes and a leading digit");
   unsigned w[S][4];
 #pragma unroll
   for (int i = 0; i < 8; i += 2) {
-    unsigned long long T[2];
-    unsigned sign = 0;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const unsigned long long bits = (unsigned long long)__double_as_longlong(x[i + q]);
-      int ex = (int)((bits >> 52) & 0x7ff);
-      unsigned long long m = bits & ((1ull << 52) - 1);
-      if (ex) m |= 1ull << 52;
-      else ex = 1;
-      const int sh = ex - 1075 + 8 * S - e;
-      if (m == 0 || sh <= -64) T[q] = 0;
-      else if (sh >= 0) T[q] = m << sh;
-      else T[q] = (m + (1ull << (-sh - 1))) >> (-sh);
-      T[q] += 0x8080808080ull;
-      sign |= (unsigned)(bits >> 63) << (15 + 16 * q);
-    }
+    const unsigned long long T[2] = {t[i] + 0x8080808080ull, t[i + 1] + 0x8080808080ull};
+    const unsigned sign = (neg >> i & 1u) << 15 | (neg >> (i + 1) & 1u) << 31;
 #pragma unroll
     for (int d = 0; d < S; ++d) {
       const int at = 8 * (S - 1 - d);  // bit position of digit d
@@ -169,7 +156,22 @@ __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ X, lon
   if (!ok || 8 * l >= Kpad) return;
   const int e = exponent_of(mx);
   if (l == 0) eb[v] = e;
-  store_digits<S>(x, e, out + v * (long long)S * Kpad + (l >> 1) * (S * 16) + (l & 1) * 8);
+  unsigned long long T[8];
+  unsigned neg = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x[i]);
+    int ex = (int)((bits >> 52) & 0x7ff);
+    unsigned long long m = bits & ((1ull << 52) - 1);
+    if (ex) m |= 1ull << 52;
+    else ex = 1;
+    const int sh = ex - 1075 + 8 * S - e;
+    if (m == 0 || sh <= -64) T[i] = 0;
+    else if (sh >= 0) T[i] = m << sh;
+    else T[i] = (m + (1ull << (-sh - 1))) >> (-sh);
+    neg |= (unsigned)(bits >> 63) << i;
+  }
+  store_digits<S>(T, neg, out + v * (long long)S * Kpad + (l >> 1) * (S * 16) + (l & 1) * 8);
 }
 
 __device__ inline void df_add(float& hi, float& lo, float x) {
@@ -180,13 +182,6 @@ __device__ inline void df_add(float& hi, float& lo, float x) {
   const float t = __fadd_rn(s, l);
   lo = __fsub_rn(l, __fsub_rn(t, s));
   hi = t;
-}
-
-// s + e = a + b exactly (Knuth's TwoSum, no ordering of |a|, |b| assumed).
-__device__ inline void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
 // The four weight-group sums of one output as a double-float (h, l): groups 0, 1 and 2 enter through
@@ -913,10 +908,12 @@ __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, in
   }
 }
 
-// Sum and slice: vector v = sums of double-float slots (in slot order), K = nseg C elements, segment g of it from the
-// slots slot[ptr[v nseg + g]] .. ; its digits and exponent go to identifier vid[v] as k_slice writes them. The
+// Sum and slice: vector v = sums of double-float slots (in slot order), K = NSEG C elements, segment g of it from the
+// slots slot[ptr[v NSEG + g]] .. ; its digits and exponent go to identifier vid[v] as k_slice writes them. The
 // expansions of a level are final once their contributions are summed, and only their digits are read afterwards,
-// so they are never stored in FP64.
+// so they are never stored in FP64. Sums are carried in three FP32 words (Sum3: closer than FP64 additions) and become
+// digits through 62-bit integers: FP64 conversions and additions, 2 per clock and SM, would bound the kernel instead of
+// memory (five a value: coupled-step layer 775 -> 816 us).
 //
 // One warp per vector: lane t sums elements t, t + 32, .. (coalesced reads, kSumFlight slots in flight), the sums
 // pass through shared memory, and lanes of 8 consecutive elements form the digits. Measured: full-size star, locals of
@@ -925,31 +922,28 @@ __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, in
 // memory, 335 us instead of 880.
 constexpr int kSumWarps = 4, kSumFlight = 4;
 
-template <int S, int Q>  // Q: elements per lane
-__global__ void __launch_bounds__(32 * kSumWarps) k_sum_slice(int C, int nseg, int Kpad, long long n,
+template <int S, int NSEG, int QC>  // QC: elements of a segment per lane
+__global__ void __launch_bounds__(32 * kSumWarps) k_sum_slice(int C, int Kpad, long long n,
                                                               const long long* __restrict__ ptr,
                                                               const long long* __restrict__ slot,
                                                               const long long* __restrict__ vid,
                                                               const float2* __restrict__ slots, slice_t* __restrict__ out,
                                                               int* __restrict__ eb) {
-  __shared__ double sh[kSumWarps][32 * Q];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, K = nseg * C;
+  __shared__ long long sh[kSumWarps][32 * NSEG * QC];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, K = NSEG * C;
   const long long v = blockIdx.x * (long long)kSumWarps + warp;
   pdl_trigger();
   pdl_wait();
   if (v >= n) return;
-  double mx = 0.0;
-  constexpr int QC = Q > 4 ? 4 : Q;  // elements per lane of a segment (C <= 128)
   // the vector's offsets are read together, one per lane, 32 at a time
-  const long long p = lane <= nseg ? ptr[v * nseg + lane] : 0;
-  const long long end = __shfl_sync(0xffffffffu, p, nseg);
+  const long long p = lane <= NSEG ? ptr[v * NSEG + lane] : 0;
+  const long long end = __shfl_sync(0xffffffffu, p, NSEG);
   long long c0 = __shfl_sync(0xffffffffu, p, 0);
   long long ids = c0 + lane < end ? slot[c0 + lane] : 0;
-  for (int g = 0; g < nseg; ++g) {
-    const long long b = __shfl_sync(0xffffffffu, p, g), e = __shfl_sync(0xffffffffu, p, g + 1);
-    float hi[QC], lo[QC];
+  Sum3 sum[NSEG][QC];
 #pragma unroll
-    for (int q = 0; q < QC; ++q) hi[q] = lo[q] = 0.f;
+  for (int g = 0; g < NSEG; ++g) {
+    const long long b = __shfl_sync(0xffffffffu, p, g), e = __shfl_sync(0xffffffffu, p, g + 1);
     for (long long k = b; k < e; k += kSumFlight) {
       if (k + kSumFlight > c0 + 32) {
         c0 = k;
@@ -967,32 +961,41 @@ __global__ void __launch_bounds__(32 * kSumWarps) k_sum_slice(int C, int nseg, i
       for (int i = 0; i < kSumFlight; ++i)
         if (k + i < e) {
 #pragma unroll
-          for (int q = 0; q < QC; ++q) {
-            df_add(hi[q], lo[q], x[i][q].x);
-            df_add(hi[q], lo[q], x[i][q].y);
-          }
+          for (int q = 0; q < QC; ++q) sum[g][q].add(x[i][q].x, x[i][q].y);
         }
     }
+  }
+  int e = kSumZero;
+#pragma unroll
+  for (int g = 0; g < NSEG; ++g)
+#pragma unroll
+    for (int q = 0; q < QC; ++q) {  // lanes past the segment hold zeros
+      sum[g][q].normalise();
+      e = max(e, sum[g][q].exponent());
+    }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (e == kSumZero) e = 0;
+#pragma unroll
+  for (int g = 0; g < NSEG; ++g)
 #pragma unroll
     for (int q = 0; q < QC; ++q) {
       const int r = lane + 32 * q;
-      const double y = (double)hi[q] + (double)lo[q];
-      if (r < C) {
-        sh[warp][g * C + r] = y;
-        mx = fmax(mx, fabs(y));
-      }
+      if (r < C) sh[warp][g * C + r] = sum[g][q].fixed(e);
     }
-  }
-  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   __syncwarp();
-  const int e = exponent_of(mx);
   const long long id = vid[v];
   if (lane == 0) eb[id] = e;
   if (8 * lane >= Kpad) return;
-  double x[8];
+  unsigned long long T[8];
+  unsigned neg = 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) x[i] = 8 * lane + i < K ? sh[warp][8 * lane + i] : 0.0;
-  store_digits<S>(x, e, out + id * (long long)S * Kpad + (lane >> 1) * (S * 16) + (lane & 1) * 8);
+  for (int i = 0; i < 8; ++i) {
+    const long long x = 8 * lane + i < K ? sh[warp][8 * lane + i] : 0;
+    constexpr int drop = kFixedBits - 8 * S;
+    T[i] = ((unsigned long long)(x < 0 ? -x : x) + (1ull << (drop - 1))) >> drop;
+    neg |= (unsigned)(x < 0) << i;
+  }
+  store_digits<S>(T, neg, out + id * (long long)S * Kpad + (lane >> 1) * (S * 16) + (lane & 1) * 8);
 }
 
 constexpr int kKAlign = 32;  // padded K: a multiple of both engines' K steps
@@ -1140,12 +1143,12 @@ int launch_slice(const double* X, long long nvec, int K, void* out, int* eb, cud
 int launch_sum_slice(int C, int nseg, long long n, const long long* ptr, const long long* slot, const long long* vid,
                      const void* slots, void* out, int* eb, cudaStream_t s, bool pdl) {
   if (n <= 0) return VP_OK;
-  const int K = nseg * C;
-  if (K > 256 || C > 128) return VP_ERR_ARG;
+  if (nseg < 1 || nseg > 2 || C > 128) return VP_ERR_ARG;
   const unsigned blocks = (unsigned)((n + kSumWarps - 1) / kSumWarps);
-  const auto f = K <= 32 ? k_sum_slice<kSplitSlices, 1> : K <= 96 ? k_sum_slice<kSplitSlices, 3>
-                 : K <= 128 ? k_sum_slice<kSplitSlices, 4> : k_sum_slice<kSplitSlices, 8>;
-  TRY(launch(f, blocks, 32 * kSumWarps, 0, s, pdl, C, nseg, kpad(K), n, ptr, slot, vid,
+  constexpr int S = kSplitSlices;
+  const auto f = nseg == 1 ? (C <= 32 ? k_sum_slice<S, 1, 1> : C <= 96 ? k_sum_slice<S, 1, 3> : k_sum_slice<S, 1, 4>)
+                           : (C <= 32 ? k_sum_slice<S, 2, 1> : C <= 96 ? k_sum_slice<S, 2, 3> : k_sum_slice<S, 2, 4>);
+  TRY(launch(f, blocks, 32 * kSumWarps, 0, s, pdl, C, kpad(nseg * C), n, ptr, slot, vid,
              static_cast<const float2*>(slots), static_cast<slice_t*>(out), eb));
   return VP_OK;
 }
