@@ -229,27 +229,52 @@ __global__ void k_layout(int Cin, int Cout, int K, const float* __restrict__ p, 
 }
 
 // Part sums of dW[o][c][k] = sum_{b,x} dz[b][o][x] a[b][c][(x + k - K/2) mod n] and dbias[o] = sum dz over a
-// segment of the positions: block (seg, o tile, c tile) takes every gridDim.x-th chunk of kWX positions.
+// segment of the positions: block (seg, pair) takes every gridDim.x-th chunk of kWX positions for the pair0 + pair-th
+// pair of an output and an input channel tile.
 // A thread holds OT output channels x 2 input channels x K taps in registers and walks along x four positions at a
 // time, so an input position is read once for its K taps: with OT = 4 and K = 9, 10 shared reads of 16 bytes for
 // 288 multiply-adds (one (o, c) pair per block read 10 values from L1 per 10 multiply-adds). Chunks are copied
 // to shared memory one ahead (cp.async). Row pitches of 4 mod 32 words and channels dealt out row by row keep
-// the reads free of bank conflicts. part[seg][Cout Cin K + Cout] is summed by k_sum_parts, so the result does
-// not depend on the order in which blocks run.
+// the reads free of bank conflicts. part[seg][pair][output][input channel][tap], then [output] for the bias, is summed
+// by k_sum_parts, so the result does not depend on the order in which blocks run.
+// SHORT: eight products are added up before they enter a running sum, which keeps its chain to 8 and its error to that of
+// one term per thread and a tree over the threads; it costs an eighth more instructions (batch 32, n = 4096: 1,806 instead
+// of 1,666 us for the gradient), so longer sums, whose single chains of B n / 304 products stay below
+// the B n / 256 of 256 threads, do without.
 // Measured (64 x 64 channels, K = 9, n = 4096, batch 32): 227 us = 43 TFLOP/s, FP32 pipe 58 % busy, 13 us for the
 // sum (about 3.3 ms with a block per (o, c) pair).
 constexpr int kWX = 64;                   // positions per chunk
 constexpr int kWPitchZ = kWX + 4;         // row of the dz chunk
 constexpr int kWPitchA = kWX + 20;        // row of the activation chunk (halos of at most 8 on each side)
 
-template <int K, int OT>
+// Output channels held by a thread (at most 72 sums) and of a tile; the tiles of a layer and their share of a segment's
+// part sums.
+__host__ __device__ constexpr int wgrad_ot(int K) { return K <= 9 ? 4 : 2; }
+struct WgradTiles {
+  int no, nc, pairs_c, pairs;  // channels of a tile (the layer's, if fewer), input tiles, pairs of tiles
+  size_t ld;                   // part sums of a pair
+};
+WgradTiles wgrad_tiles(int Cin, int Cout, int K) {
+  const int ot = 16 * wgrad_ot(K);
+  WgradTiles t;
+  t.no = std::min(Cout, ot);
+  t.nc = std::min(Cin, kTO);
+  t.pairs_c = (Cin + kTO - 1) / kTO;
+  t.pairs = (Cout + ot - 1) / ot * t.pairs_c;
+  t.ld = (size_t)t.no * t.nc * K + t.no;
+  return t;
+}
+
+template <int K, bool SHORT>
 __global__ void __launch_bounds__(512) k_conv_wgrad(int n, int B, int Cin, int Cout, const float* __restrict__ dz,
                                                     const float* __restrict__ a, float* __restrict__ part,
-                                                    size_t part_ld, int vec) {
+                                                    WgradTiles tl, int pair0, int vec) {
   extern __shared__ __align__(16) float wg_sm[];
-  constexpr int half = K / 2, PAD = halo(K), off = PAD - half, NW = (off + K + 6) / 4;
+  constexpr int OT = wgrad_ot(K), half = K / 2, PAD = halo(K), off = PAD - half;
+  constexpr int kStep = SHORT ? 8 : 4, NW = (off + K + kStep + 2) / 4;  // positions of a step; 16-byte reads per window
   constexpr int kOTile = 16 * OT;
-  const int o0 = blockIdx.y * kOTile, c0 = blockIdx.z * kTO;
+  const int ot = (pair0 + (int)blockIdx.y) / tl.pairs_c, ct = (pair0 + (int)blockIdx.y) - ot * tl.pairs_c;
+  const int o0 = ot * kOTile, c0 = ct * kTO;
   const int no = min(kOTile, Cout - o0), nc = min(kTO, Cin - c0);
   const int nog = (no + OT - 1) / OT, ncg = (nc + 1) / 2;
   const int zrows = nog * OT, arows = ncg * 2;
@@ -290,13 +315,8 @@ __global__ void __launch_bounds__(512) k_conv_wgrad(int n, int B, int Cin, int C
     const float* sa = sz + zrows * kWPitchZ;
     if (live) {
 #pragma unroll 1
-      for (int x = 0; x < kWX; x += 4) {
-        float d[OT][4], w[2][NW * 4];
-#pragma unroll
-        for (int r = 0; r < OT; ++r) {
-          const float4 v = *reinterpret_cast<const float4*>(sz + (og + r * nog) * kWPitchZ + x);
-          d[r][0] = v.x; d[r][1] = v.y; d[r][2] = v.z; d[r][3] = v.w;
-        }
+      for (int x = 0; x < kWX; x += kStep) {
+        float w[2][NW * 4];
 #pragma unroll
         for (int q = 0; q < 2; ++q)
 #pragma unroll
@@ -305,26 +325,35 @@ __global__ void __launch_bounds__(512) k_conv_wgrad(int n, int B, int Cin, int C
             w[q][4 * t] = v.x; w[q][4 * t + 1] = v.y; w[q][4 * t + 2] = v.z; w[q][4 * t + 3] = v.w;
           }
 #pragma unroll
-        for (int t = 0; t < 4; ++t)
+        for (int r = 0; r < OT; ++r) {
+          float d[kStep];
 #pragma unroll
-          for (int r = 0; r < OT; ++r)
+          for (int t = 0; t < kStep; t += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(sz + (og + r * nog) * kWPitchZ + x + t);
+            d[t] = v.x; d[t + 1] = v.y; d[t + 2] = v.z; d[t + 3] = v.w;
+          }
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
+          for (int q = 0; q < 2; ++q)
 #pragma unroll
-              for (int k = 0; k < K; ++k) acc[r][q][k] = fmaf(d[r][t], w[q][off + t + k], acc[r][q][k]);
+            for (int k = 0; k < K; ++k) {
+              float s = SHORT ? 0.f : acc[r][q][k];
+#pragma unroll
+              for (int t = 0; t < kStep; ++t) s = fmaf(d[t], w[q][off + t + k], s);
+              acc[r][q][k] = SHORT ? acc[r][q][k] + s : s;
+            }
+        }
       }
     }
-    if (blockIdx.z == 0 && tid < no) {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int x = 0; x < kWX; x += 4) {
-        const float4 z = *reinterpret_cast<const float4*>(sz + tid * kWPitchZ + x);
-        v.x += z.x; v.y += z.y; v.z += z.z; v.w += z.w;
+    if (ct == 0 && tid < no) {
+      for (int x = 0; x < kWX; x += 8) {
+        const float4 y = *reinterpret_cast<const float4*>(sz + tid * kWPitchZ + x);
+        const float4 z = *reinterpret_cast<const float4*>(sz + tid * kWPitchZ + x + 4);
+        bsum += ((y.x + y.y) + (y.z + y.w)) + ((z.x + z.y) + (z.z + z.w));
       }
-      bsum += (v.x + v.y) + (v.z + v.w);
     }
     __syncthreads();
   }
-  float* pw = part + (size_t)blockIdx.x * part_ld;
+  float* pw = part + ((size_t)blockIdx.x * gridDim.y + blockIdx.y) * tl.ld;
   if (live) {
 #pragma unroll
     for (int r = 0; r < OT; ++r)
@@ -333,33 +362,32 @@ __global__ void __launch_bounds__(512) k_conv_wgrad(int n, int B, int Cin, int C
         const int o = og + r * nog, c = cg + q * ncg;
         if (o < no && c < nc)
 #pragma unroll
-          for (int k = 0; k < K; ++k) pw[((size_t)(o0 + o) * Cin + c0 + c) * K + k] = acc[r][q][k];
+          for (int k = 0; k < K; ++k) pw[((size_t)o * tl.nc + c) * K + k] = acc[r][q][k];
       }
   }
-  if (blockIdx.z == 0 && tid < no) pw[(size_t)Cout * Cin * K + o0 + tid] = bsum;
+  if (ct == 0 && tid < no) pw[(size_t)tl.no * tl.nc * K + tid] = bsum;
 }
 
 size_t wgrad_smem(int zrows, int arows) { return (size_t)2 * (zrows * kWPitchZ + arows * kWPitchA) * sizeof(float); }
 
+// Pairs pair0 .. pair0 + pairs - 1 of the layer's tiles.
 template <int K>
 int launch_wgrad_k(int n, int B, int Cin, int Cout, const float* dz, const float* a, float* part, int segs,
-                   cudaStream_t s) {
-  constexpr int OT = K <= 9 ? 4 : 2, kOTile = 16 * OT;  // at most 72 sums per thread
-  const int no = std::min(Cout, kOTile), nc = std::min(Cin, kTO);
-  const int nog = (no + OT - 1) / OT, ncg = (nc + 1) / 2;
+                   const WgradTiles& tl, int pair0, int pairs, cudaStream_t s) {
+  constexpr int OT = wgrad_ot(K);
+  const int nog = (tl.no + OT - 1) / OT, ncg = (tl.nc + 1) / 2;
   const int threads = std::max(64, (nog * ncg + 31) / 32 * 32);  // a thread per output channel for the bias sums
-  k_conv_wgrad<K, OT><<<dim3(segs, (Cout + kOTile - 1) / kOTile, (Cin + kTO - 1) / kTO), threads,
-                        wgrad_smem(nog * OT, ncg * 2), s>>>(n, B, Cin, Cout, dz, a, part,
-                                                            (size_t)Cout * Cin * K + Cout,
-                                                            n % 4 == 0 && aligned16(dz) && aligned16(a));
+  const bool one_chunk = (long long)B * ((n + kWX - 1) / kWX) == segs;
+  (one_chunk ? k_conv_wgrad<K, true> : k_conv_wgrad<K, false>)<<<dim3(segs, pairs), threads, wgrad_smem(nog * OT, ncg * 2), s>>>(
+      n, B, Cin, Cout, dz, a, part, tl, pair0, n % 4 == 0 && aligned16(dz) && aligned16(a));
   TRY(cudaGetLastError());
   return VP_OK;
 }
 
 template <int K>
 int prepare_k() {
-  TRY(cudaFuncSetAttribute(k_conv_wgrad<K, (K <= 9 ? 4 : 2)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)wgrad_smem(kTO, kTO)));
+  for (auto f : {k_conv_wgrad<K, true>, k_conv_wgrad<K, false>})
+    TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_smem(kTO, kTO)));
   TRY(cudaFuncSetAttribute(k_conv<K, 1, 1, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem<K, 1, 16>()));
   TRY(cudaFuncSetAttribute(k_conv<K, 8, 2, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem<K, 2, 16>()));
   TRY(cudaFuncSetAttribute(k_conv<K, 4, 1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem<K, 1, 8>()));
@@ -382,17 +410,24 @@ auto conv_of(int k) -> decltype(&launch_conv_k<1>) { WS_BY_K(k, launch_conv_k) }
 auto wgrad_of(int k) -> decltype(&launch_wgrad_k<1>) { WS_BY_K(k, launch_wgrad_k) }
 auto prepare_of(int k) -> decltype(&prepare_k<1>) { WS_BY_K(k, prepare_k) }
 
-// Segments of a weight gradient: two blocks per SM of the 152 for the widest layers (an uneven last wave costs
-// less, and the running sums are half as long as with one), as far as the part sums fit kPartBytes.
+// Segments of a weight gradient: two blocks per SM of the 152 (an uneven last wave costs less, and the running sums are
+// half as long as with one), whatever the layer's width: tiles beyond kPartBytes of part sums take their turns
+// (one pair of tiles takes 45 MB at most). Fewer segments for wider layers made the sums longer: at 512 x 512 channels,
+// K = 15, 2048 positions the gradient's error was 1.08e-7 with 8 segments and single running sums, 6.2e-8 with a tree
+// over 256 threads, 4.6e-8 now.
+// No more segments than chunks: the sums over empty ones cost a network of 4 channels 73 -> 85 us a gradient.
 constexpr int kMaxSegs = 304;
+int wgrad_segs(int n, int B) { return (int)std::min<long long>(kMaxSegs, (long long)B * ((n + kWX - 1) / kWX)); }
 constexpr size_t kPartBytes = (size_t)128 << 20;
-int wgrad_segs(size_t layer_params) {
-  return (int)std::max<size_t>(1, std::min<size_t>(kMaxSegs, kPartBytes / (layer_params * sizeof(float))));
+size_t part_floats(const WgradTiles& tl, int segs) {
+  const size_t one = segs * tl.ld;
+  return one * std::max<size_t>(1, std::min<size_t>(tl.pairs, kPartBytes / sizeof(float) / one));
 }
 
-// g[p] = sum over the segments of part[seg][p], compensated: 32 parameters per block, warp w taking the
-// segments w mod 8, the eight sums added in their order.
-__global__ void __launch_bounds__(256) k_sum_parts(size_t m, int segs, const float* __restrict__ part, float* __restrict__ g) {
+// Sums over the segments of part[seg][m], compensated, into the layer's gradient g (weights [output][input][tap], then
+// the bias): 32 part sums per block, warp w taking the segments w mod 8, the eight sums added in their order.
+__global__ void __launch_bounds__(256) k_sum_parts(size_t m, int segs, const float* __restrict__ part, WgradTiles tl,
+                                                   int pair0, int Cin, int Cout, int K, float* __restrict__ g) {
   __shared__ float2 sh[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t p = blockIdx.x * (size_t)32 + lane;
@@ -413,7 +448,17 @@ __global__ void __launch_bounds__(256) k_sum_parts(size_t m, int segs, const flo
     add(sh[q][lane].x);
     e += sh[q][lane].y;
   }
-  g[p] = s + e;
+  const int pair = pair0 + (int)(p / tl.ld), ot = pair / tl.pairs_c, ct = pair - ot * tl.pairs_c;
+  int r = (int)(p % tl.ld);
+  const int weights = tl.no * tl.nc * K, o = ot * 16 * wgrad_ot(K) + (r < weights ? r / (tl.nc * K) : r - weights);
+  if (o >= Cout) return;
+  if (r < weights) {
+    r %= tl.nc * K;
+    const int c = ct * kTO + r / K;
+    if (c < Cin) g[((size_t)o * Cin + c) * K + r % K] = s + e;
+  } else if (ct == 0) {
+    g[(size_t)Cout * Cin * K + o] = s + e;
+  }
 }
 
 // g = 2 (y - t) / m and partial sums of (y - t)^2 (one per block, into part[blockIdx.x]).
@@ -461,7 +506,8 @@ struct ws_s {
   std::vector<float*> act;                  // activations a_0..a_{L-1}, z_L (size L+1), max_batch each
   float *d0 = nullptr, *d1 = nullptr;       // gradient work buffers
   double* part = nullptr;
-  float* wparts = nullptr;                  // part sums of one layer's weight gradient
+  float* wparts = nullptr;                  // part sums of a layer's weight gradient, or of some of its tiles
+  size_t part_count = 0;                    // elements of wparts
   long long step = 0;
   std::vector<void*> allocs;
 };
@@ -524,11 +570,17 @@ int grad(ws_s* w, const float* x, const float* t, int B, float* loss, cudaStream
   for (int l = w->L - 1; l >= 0; --l) {
     const int Cin = w->C[l], Cout = w->C[l + 1];
     const float* a = (l == 0) ? x : w->act[l];
-    const size_t m = (size_t)Cout * Cin * w->K + Cout;  // weights, then bias
-    const int segs = wgrad_segs(m);
-    if ((rc = wgrad_of(w->K)(w->n, B, Cin, Cout, dz, a, w->wparts, segs, s))) return rc;
-    k_sum_parts<<<(unsigned)((m + 31) / 32), 256, 0, s>>>(m, segs, w->wparts, w->g + w->woff[l]);
-    TRY(cudaGetLastError());
+    const WgradTiles tl = wgrad_tiles(Cin, Cout, w->K);
+    const int segs = wgrad_segs(w->n, B);
+    const int group = (int)std::min<size_t>({(size_t)tl.pairs, w->part_count / (segs * tl.ld), 65535});
+    for (int pair0 = 0; pair0 < tl.pairs; pair0 += group) {
+      const int pairs = std::min(group, tl.pairs - pair0);
+      if ((rc = wgrad_of(w->K)(w->n, B, Cin, Cout, dz, a, w->wparts, segs, tl, pair0, pairs, s))) return rc;
+      const size_t m = pairs * tl.ld;
+      k_sum_parts<<<(unsigned)((m + 31) / 32), 256, 0, s>>>(m, segs, w->wparts, tl, pair0, Cin, Cout, w->K,
+                                                            w->g + w->woff[l]);
+      TRY(cudaGetLastError());
+    }
     if (l > 0) {
       // da masked by the activation of the layer
       if ((rc = conv_of(w->K)(w->n, B, Cout, Cin, w->wb[l], nullptr, dz, da, 0, w->act[l], s))) return rc;
@@ -597,9 +649,9 @@ extern "C" int ws_create(int in_ch, int width, int out_ch, int n_layers, int ksi
     if (cudaMemsetAsync(w->wf[l], 0, nf * sizeof(float), s) != cudaSuccess ||
         cudaMemsetAsync(w->wb[l], 0, nb * sizeof(float), s) != cudaSuccess)
       return fail(VP_ERR_CUDA);
-    const size_t m = (size_t)w->C[l + 1] * w->C[l] * ksize + w->C[l + 1];
-    parts = std::max(parts, m * wgrad_segs(m));
+    parts = std::max(parts, part_floats(wgrad_tiles(w->C[l], w->C[l + 1], ksize), wgrad_segs(n, max_batch)));
   }
+  w->part_count = parts;
   if ((rc = walloc(w.get(), &w->wparts, parts)) || (rc = prepare_of(ksize)())) return fail(rc);
   {
     void* q = nullptr;
