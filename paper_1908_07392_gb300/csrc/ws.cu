@@ -71,7 +71,7 @@ __device__ inline void load_rows(float* sm, const float* src, int rows, int have
 __host__ __device__ inline int pad4(int c) { return (c + 3) & ~3; }
 
 // out[b][o][x] = (bias ? bias[o] : 0) + sum_{c,k} w(o, c, k) in[b][c][(x + k - K/2) mod n], the weights laid out as
-// W[c][k][pad4(Cout)] (k_layout); relu: max(., 0); mask (an array like out): 0 where mask is not positive.
+// W[c][k][pad4(Cout)] (Layer); relu: max(., 0); mask (an array like out): 0 where mask is not positive.
 //
 // A thread holds OT output channels x XT groups of 4 positions in registers (the groups XG * 4 apart, so that
 // the 16-byte reads of the window are free of bank conflicts). Per input channel it reads the window of
@@ -214,18 +214,35 @@ int launch_conv_k(int n, int B, int Cin, int Cout, const float* W, const float* 
   return f(n, B, Cin, Cout, W, bias, in, out, relu, mask, s);
 }
 
-// The weights of a layer ([out][in][k] in p) as k_conv reads them: wf[in][k][pad4(out)] for the forward pass, and
-// wb[out][k][pad4(in)], reversed in k, for the transposed convolution of the backward pass. The padding is zero from
-// the allocation on.
-__global__ void k_layout(int Cin, int Cout, int K, const float* __restrict__ p, float* __restrict__ wf,
-                         float* __restrict__ wb) {
-  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;  // layers of 2^31 weights and more are accepted
-  if (e >= (size_t)Cin * Cout * K) return;
-  const int c = (int)(e / K % Cin), k = (int)(e % K);
-  const size_t o = e / K / Cin;
-  const float v = p[e];
-  wf[((size_t)c * K + k) * pad4(Cout) + o] = v;
-  wb[(o * K + K - 1 - k) * pad4(Cin) + c] = v;
+// The weights of a layer ([out][in][k] at woff in the parameters, the bias at boff) as k_conv reads them:
+// wf[in][k][pad4(out)] for the forward pass, and wb[out][k][pad4(in)], reversed in k, for the transposed convolution of
+// the backward pass. The padding is zero from the allocation on.
+struct Layer {
+  size_t woff, boff;
+  int Cin, Cout;
+  float *wf, *wb;
+};
+
+// Parameter e, now v, into its layer's layouts.
+__device__ inline void store_layouts(const Layer* __restrict__ layers, int L, int K, size_t e, float v) {
+  int l = 0;
+  for (int hi = L - 1; l < hi;) {
+    const int mid = (l + hi + 1) / 2;
+    if (layers[mid].woff <= e) l = mid;
+    else hi = mid - 1;
+  }
+  const Layer y = layers[l];
+  if (e >= y.boff) return;  // a bias
+  e -= y.woff;              // layers of 2^31 weights and more are accepted
+  const int c = (int)(e / K % y.Cin), k = (int)(e % K);
+  const size_t o = e / K / y.Cin;
+  y.wf[((size_t)c * K + k) * pad4(y.Cout) + o] = v;
+  y.wb[(o * K + K - 1 - k) * pad4(y.Cin) + c] = v;
+}
+
+__global__ void k_layouts(const Layer* __restrict__ layers, int L, int K, size_t m, const float* __restrict__ p) {
+  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (e < m) store_layouts(layers, L, K, e, p[e]);
 }
 
 // Part sums of dW[o][c][k] = sum_{b,x} dz[b][o][x] a[b][c][(x + k - K/2) mod n] and dbias[o] = sum dz over a
@@ -481,8 +498,11 @@ __global__ void k_mse(size_t m, const float* __restrict__ y, const float* __rest
   }
 }
 
+// Adam, and the layouts of the new weights (a launch per layer for them took a step of three small layers from 93 to
+// 110 us).
 __global__ void k_adam(size_t m, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ mo,
-                       float* __restrict__ ve, float lr, float b1, float b2, float eps, float c1, float c2) {
+                       float* __restrict__ ve, float lr, float b1, float b2, float eps, float c1, float c2,
+                       const Layer* __restrict__ layers, int L, int K) {
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i >= m) return;
   const float gi = g[i];
@@ -490,7 +510,9 @@ __global__ void k_adam(size_t m, float* __restrict__ p, const float* __restrict_
   const float vi = b2 * ve[i] + (1.f - b2) * gi * gi;
   mo[i] = mi;
   ve[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  const float v = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  p[i] = v;
+  store_layouts(layers, L, K, i, v);
 }
 
 }  // namespace
@@ -502,7 +524,8 @@ struct ws_s {
   std::vector<size_t> woff, boff;           // parameter offsets
   size_t nparams = 0;
   float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
-  std::vector<float*> wf, wb;               // per layer: the weights as k_conv reads them (k_layout)
+  std::vector<float*> wf, wb;               // per layer: the weights as k_conv reads them (Layer)
+  vp::Layer* layers = nullptr;                  // the same on the device
   std::vector<float*> act;                  // activations a_0..a_{L-1}, z_L (size L+1), max_batch each
   float *d0 = nullptr, *d1 = nullptr;       // gradient work buffers
   double* part = nullptr;
@@ -532,14 +555,10 @@ inline uint64_t splitmix64(uint64_t& s) {
   return z ^ (z >> 31);
 }
 
-// The convolution layouts of the weights, after every change of the parameters.
+// The convolution layouts of the weights, after the parameters have been replaced.
 int layout(ws_s* w, cudaStream_t s) {
-  for (int l = 0; l < w->L; ++l) {
-    const int Cin = w->C[l], Cout = w->C[l + 1];
-    k_layout<<<(unsigned)(((size_t)Cin * Cout * w->K + 255) / 256), 256, 0, s>>>(Cin, Cout, w->K, w->p + w->woff[l],
-                                                                              w->wf[l], w->wb[l]);
-    TRY(cudaGetLastError());
-  }
+  k_layouts<<<(unsigned)((w->nparams + 255) / 256), 256, 0, s>>>(w->layers, w->L, w->K, w->nparams, w->p);
+  TRY(cudaGetLastError());
   return VP_OK;
 }
 
@@ -572,13 +591,15 @@ int grad(ws_s* w, const float* x, const float* t, int B, float* loss, cudaStream
     const float* a = (l == 0) ? x : w->act[l];
     const WgradTiles tl = wgrad_tiles(Cin, Cout, w->K);
     const int segs = wgrad_segs(w->n, B);
+    const bool direct = segs == 1 && tl.pairs == 1;  // the one tile's part sums are the gradient, in its order
     const int group = (int)std::min<size_t>({(size_t)tl.pairs, w->part_count / (segs * tl.ld), 65535});
+    float* g = w->g + w->woff[l];
     for (int pair0 = 0; pair0 < tl.pairs; pair0 += group) {
       const int pairs = std::min(group, tl.pairs - pair0);
-      if ((rc = wgrad_of(w->K)(w->n, B, Cin, Cout, dz, a, w->wparts, segs, tl, pair0, pairs, s))) return rc;
+      if ((rc = wgrad_of(w->K)(w->n, B, Cin, Cout, dz, a, direct ? g : w->wparts, segs, tl, pair0, pairs, s))) return rc;
+      if (direct) break;
       const size_t m = pairs * tl.ld;
-      k_sum_parts<<<(unsigned)((m + 31) / 32), 256, 0, s>>>(m, segs, w->wparts, tl, pair0, Cin, Cout, w->K,
-                                                            w->g + w->woff[l]);
+      k_sum_parts<<<(unsigned)((m + 31) / 32), 256, 0, s>>>(m, segs, w->wparts, tl, pair0, Cin, Cout, w->K, g);
       TRY(cudaGetLastError());
     }
     if (l > 0) {
@@ -653,11 +674,18 @@ extern "C" int ws_create(int in_ch, int width, int out_ch, int n_layers, int ksi
   }
   w->part_count = parts;
   if ((rc = walloc(w.get(), &w->wparts, parts)) || (rc = prepare_of(ksize)())) return fail(rc);
+  std::vector<Layer> layers(n_layers);
+  for (int l = 0; l < n_layers; ++l) layers[l] = {w->woff[l], w->boff[l], w->C[l], w->C[l + 1], w->wf[l], w->wb[l]};
   {
-    void* q = nullptr;
+    void *q = nullptr, *d = nullptr;
     if (cudaMalloc(&q, 256 * sizeof(double)) != cudaSuccess) return fail(VP_ERR_OOM);
     w->allocs.push_back(q);
     w->part = static_cast<double*>(q);
+    if (cudaMalloc(&d, layers.size() * sizeof(Layer)) != cudaSuccess) return fail(VP_ERR_OOM);
+    w->allocs.push_back(d);
+    w->layers = static_cast<Layer*>(d);
+    if (cudaMemcpyAsync(d, layers.data(), layers.size() * sizeof(Layer), cudaMemcpyHostToDevice, s) != cudaSuccess)
+      return fail(VP_ERR_CUDA);
   }
   // initial parameters: uniform in +-1/sqrt(fan_in) from a seeded splitmix64 stream
   std::vector<float> host(off);
@@ -721,7 +749,7 @@ extern "C" int ws_train_step(ws_net net, const float* x, const float* t, int bat
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - std::pow(b1, (float)net->step), c2 = 1.f - std::pow(b2, (float)net->step);
   k_adam<<<(unsigned)((net->nparams + 255) / 256), 256, 0, s>>>(net->nparams, net->p, net->g, net->m, net->v, lr, b1,
-                                                                 b2, 1e-8f, c1, c2);
+                                                                 b2, 1e-8f, c1, c2, net->layers, net->L, net->K);
   TRY(cudaGetLastError());
-  return layout(net, s);
+  return VP_OK;
 }
