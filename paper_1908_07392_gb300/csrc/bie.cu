@@ -593,24 +593,24 @@ __global__ void __launch_bounds__(256) k_gm_backsub(int m, const GmresCtl* ctl, 
   }
 }
 
-// u(x_t) = sum_j D(x_t, y_j) mu_j w_j (targets away from the boundary), two targets per block.
+// u(x_t) = sum_j D(x_t, y_j) mu_j w_j (targets away from the boundary), NT targets per block.
 //
 // FP64 bounds it. For alpha r >= kFarZ the terms of T1, T2, T3 with K0 and K1 are below 2^-54 of the algebraic
 // ones (z^3 e^-z sqrt(pi / 2z) < 5e-18 against 4), so adding them changes nothing and only the algebraic part is
 // formed: with q = 1 / r^2, c = 2 q^2 / (pi alpha^2), m = mu w,
 //   D m = -c (n (r.m) + r (n.m) + m (r.n)) + 4 c q r (r.n)(r.m) + q / (2 pi) r (n.m),
-// about 35 FP64 operations and no transcendental function. Measured: 2000 targets, 4096 nodes, alpha = 316: 563 us
-// (5,743 us with the Bessel functions for every pair).
+// about 35 FP64 operations and no transcendental function. Measured: 2000 targets, 4096 nodes, alpha = 316: 576 us
+// (5,754 us with the Bessel functions for every pair).
 constexpr double kFarZ = 50.0;
-constexpr int kEvalTargets = 2;
 
+template <int NT>
 __global__ void __launch_bounds__(256) k_eval_dl(int N, double alpha, Nodes nd, const double* mu, int M,
                                                  const double* txy, double* u) {
-  const int t0 = blockIdx.x * kEvalTargets;
+  const int t0 = blockIdx.x * NT;
   const double far2 = kFarZ / alpha * (kFarZ / alpha), ca = 2.0 / (kPi * alpha * alpha);
-  double x[kEvalTargets], y[kEvalTargets], s[kEvalTargets][2] = {};
+  double x[NT], y[NT], s[NT][2] = {};
 #pragma unroll
-  for (int t = 0; t < kEvalTargets; ++t) {
+  for (int t = 0; t < NT; ++t) {
     const int k = min(t0 + t, M - 1);
     x[t] = txy[k];
     y[t] = txy[M + k];
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(256) k_eval_dl(int N, double alpha, Nodes nd, 
     const double xj = nd.x[j], yj = nd.y[j], nx = nd.nx[j], ny = nd.ny[j], w = nd.w[j];
     const double mx = mu[2 * j] * w, my = mu[2 * j + 1] * w, nm = nx * mx + ny * my;
 #pragma unroll
-    for (int t = 0; t < kEvalTargets; ++t) {
+    for (int t = 0; t < NT; ++t) {
       const double rx = x[t] - xj, ry = y[t] - yj, r2 = rx * rx + ry * ry;
       if (r2 >= far2) {
         const double q = 1.0 / r2, c = ca * q * q;
@@ -635,9 +635,9 @@ __global__ void __launch_bounds__(256) k_eval_dl(int N, double alpha, Nodes nd, 
       }
     }
   }
-  __shared__ double red[8][2 * kEvalTargets];
+  __shared__ double red[8][2 * NT];
 #pragma unroll
-  for (int t = 0; t < kEvalTargets; ++t)
+  for (int t = 0; t < NT; ++t)
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
       double v = s[t][a];
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(256) k_eval_dl(int N, double alpha, Nodes nd, 
       if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][2 * t + a] = v;
     }
   __syncthreads();
-  if (threadIdx.x < 2 * kEvalTargets) {
+  if (threadIdx.x < 2 * NT) {
     const int t = threadIdx.x >> 1, a = threadIdx.x & 1;
     double v = 0.0;
     for (int q = 0; q < 8; ++q) v += red[q][threadIdx.x];
@@ -698,6 +698,7 @@ struct bie_s {
   double *V = nullptr, *w = nullptr, *r = nullptr;
   double* diag = nullptr;        // the operator's diagonal; A holds the rest as digits (k_matrix_digits)
   int* re = nullptr;             // row exponents
+  int sms = 0;
   int ctas = 0, rows = 0;        // launch of k_gemv: one CTA per SM, rows of each
   double* gm = nullptr;          // H [(m+1) m], cs [m], sn [m], gv [m+2], y [m], hv [2(m+1)], scalars [8]
   double *ac = nullptr, *au = nullptr, *abv = nullptr;  // augmentation: c, u [2N], b [m]
@@ -758,8 +759,8 @@ extern "C" int bie_create(double alpha, double R, double A, int k, double phase,
   }
   int rc, dev = 0;
   TRY(cudaGetDevice(&dev));
-  TRY(cudaDeviceGetAttribute(&B->ctas, cudaDevAttrMultiProcessorCount, dev));
-  B->rows = (B->n2 + B->ctas - 1) / B->ctas;
+  TRY(cudaDeviceGetAttribute(&B->sms, cudaDevAttrMultiProcessorCount, dev));
+  B->rows = (B->n2 + B->sms - 1) / B->sms;
   B->ctas = (B->n2 + B->rows - 1) / B->rows;
   const int N = B->N;
   Nodes& nd = B->nd;
@@ -928,7 +929,15 @@ extern "C" int bie_solve(bie b, const double* g, double* mu, double tol, int max
 extern "C" int bie_eval(bie b, const double* mu, int n_targets, const double* txy, double* u, void* stream) {
   if (!b || !mu || !txy || !u || n_targets < 0) return VP_ERR_ARG;
   if (n_targets == 0) return VP_OK;
-  k_eval_dl<<<(n_targets + kEvalTargets - 1) / kEvalTargets, 256, 0, static_cast<cudaStream_t>(stream)>>>(b->N, b->alpha, b->nd, mu, n_targets, txy, u);
+  // Two targets per block share the nodes' loads (5 % of the algebraic form), where that takes no more rounds over the
+  // SMs: time goes in steps of a target per SM. Measured with one / two on 152 SMs, 4096 nodes, alpha = 30 (Bessel pairs):
+  // 100 targets 977 / 1,865 us, 400 2,790 / 3,660, 600 3,724 / 3,748, 2000 12,457 / 12,541; alpha = 316: 100 targets 60 / 99,
+  // 400 144 / 178, 600 187 / 179, 2000 605 / 576.
+  const int rounds = (n_targets + b->sms - 1) / b->sms;
+  const bool two = n_targets >= 2 * b->sms && rounds % 2 == 0;
+  const auto eval = two ? k_eval_dl<2> : k_eval_dl<1>;
+  eval<<<two ? (n_targets + 1) / 2 : n_targets, 256, 0, static_cast<cudaStream_t>(stream)>>>(b->N, b->alpha, b->nd, mu,
+                                                                                         n_targets, txy, u);
   TRY(cudaGetLastError());
   return VP_OK;
 }
