@@ -134,22 +134,33 @@ __device__ inline void store_digits(const unsigned long long (&t)[8], unsigned n
 //
 // L lanes per vector (a power of two, L >= Kpad / 8), a lane taking 8 consecutive elements: they are read once and
 // kept for the digits, and a slice of them is one 16-byte store (2-byte stores, six per element, and a second
-// read of the vector took 571 us an evaluation of the full-size star, now 459).
+// read of the vector took 571 us an evaluation of the full-size star, now 459). A warp's vectors are consecutive, so
+// they are read in order and dealt out through shared memory: X may be page-locked host memory, which lanes reading
+// their own 64 bytes piece by piece took 324 us for 4.2M elements to fetch (172 in order; 27 and 30 us from the device).
 // Measured: the star's leaf sources (40,897 vectors of 256) 79 -> 52 us = 4.0 TB/s.
 template <int S>
 __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ X, long long nvec, int K, int Kpad, int lg_l,
                                                slice_t* __restrict__ out, int* __restrict__ eb) {
-  const int L = 1 << lg_l, l = threadIdx.x & (L - 1);
-  const long long v = (blockIdx.x * 256ll + threadIdx.x) >> lg_l;
+  __shared__ double sh[8][256 + 32];  // an element of padding per 8: the lanes' reads meet no bank twice
+  const int L = 1 << lg_l, lane = threadIdx.x & 31, l = lane & (L - 1), warp = threadIdx.x >> 5;
+  const long long v0 = (blockIdx.x * 8ll + warp) << (5 - lg_l), v = v0 + (lane >> lg_l);
   const bool ok = v < nvec;
   pdl_trigger();
   pdl_wait();
+  const int count = (int)max(0ll, min(32ll >> lg_l, nvec - v0)) * K;  // at most 32 / L vectors of 8 L elements
+  const double* src = X + v0 * K;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int at = lane + 32 * i;
+    if (at < count) sh[warp][at + (at >> 3)] = src[at];
+  }
+  __syncwarp();
   double x[8];
   double mx = 0.0;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const int k = 8 * l + i;
-    x[i] = ok && k < K ? X[v * K + k] : 0.0;
+    const int k = 8 * l + i, at = (lane >> lg_l) * K + k;
+    x[i] = ok && k < K ? sh[warp][at + (at >> 3)] : 0.0;
     mx = fmax(mx, fabs(x[i]));
   }
   for (int o = L >> 1; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
