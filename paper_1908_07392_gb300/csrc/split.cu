@@ -884,7 +884,6 @@ __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, in
   const long long b = live ? a.ptr[d] : 0, e = live ? a.ptr[d + 1] : 0;
   pdl_trigger();
   pdl_wait();
-  if (!live) return;
   const float2* S = reinterpret_cast<const float2*>(a.S) + r;
   float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
   auto add = [&](float4 v) {
@@ -912,10 +911,18 @@ __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, in
     return (f == 0 ? a.u : a.g + (f - 1) * a.N) + a.dst_off[d] + (row - f * a.n);
   };
   if (vec_out) {
-    *reinterpret_cast<double2*>(out(r)) = make_double2(y0, y1);
-  } else {
-    *out(r) = y0;
-    if (r + 1 < a.M) *out(r + 1) = y1;  // may begin the next field
+    if (live) *reinterpret_cast<double2*>(out(r)) = make_double2(y0, y1);
+    return;
+  }
+  // the warp's 64 rows (one destination's: `per` is a multiple of 32) change lanes, so that each of its two stores
+  // covers 32 neighbouring rows (every second row, twice, took 156 us to page-locked host memory for
+  // 495,616 nodes of p = 11, 90 now). A row may begin the next field.
+  const int lane = threadIdx.x & 31, r0 = r - 2 * lane;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    const int from = 16 * half + (lane >> 1), row = r0 + 32 * half + lane;
+    const double e0 = __shfl_sync(0xffffffffu, y0, from), e1 = __shfl_sync(0xffffffffu, y1, from);
+    if (d < n_dst && row < a.M) *out(row) = lane & 1 ? e1 : e0;
   }
 }
 
