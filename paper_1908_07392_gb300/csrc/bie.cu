@@ -448,8 +448,8 @@ __global__ void k_gm_step(int j, int m, double tol, GmresCtl* ctl, double* H, do
 // rotations (as k_gm_step) and v_(j+1) = w / |w|; with `ac` first the projection w -= (ac . w) ac, whose
 // coefficient goes to abv[j]. A cluster of 16 CTAs holds w in shared memory, a sixteenth each; dot products meet in
 // distributed shared memory, added in the order of the ranks. The separate kernels (k_dots ... k_gm_scale) take
-// seven launches a step, each a few microseconds on a vector of 64 KB; they stay for vectors and subspaces
-// beyond kArnN and kArnCols, where more than 16 SMs' worth of FP64 pays. Measured at 8192 unknowns, 17 steps:
+// seven launches a step, each a few microseconds on a vector of 64 KB; they stay for devices that cannot hold the
+// cluster, and for vectors and subspaces beyond kArnN and kArnCols, where more than 16 SMs' worth of FP64 pays. Measured at 8192 unknowns, 17 steps:
 // 22 us a step beside the operator, 87 with the separate kernels; a cold solve 3.64 -> 2.24 ms with k_gemv.
 constexpr int kArnCtas = 16, kArnThreads = 512, kArnN = 32768, kArnCols = 64;
 
@@ -540,6 +540,25 @@ __global__ void __cluster_dims__(kArnCtas, 1, 1) __launch_bounds__(kArnThreads)
     if (res <= tol || hn == 0.0) ctl->done = 1;
   }
   cl.sync();  // no CTA ends while another reads its shared memory
+}
+
+// Whether the current device can hold a cluster of k_arnoldi, which is larger than the portable size; otherwise the
+// separate kernels take every step.
+bool arnoldi_cluster_fits() {
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(kArnCtas);
+  c.blockDim = dim3(kArnThreads);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kArnCtas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  int clusters = 0;
+  const bool ok = cudaFuncSetAttribute(k_arnoldi, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                  cudaOccupancyMaxActiveClusters(&clusters, k_arnoldi, &c) == cudaSuccess;
+  cudaGetLastError();  // not an error of the caller's
+  return ok && clusters > 0;
 }
 
 // Augmentation by a direction d (w = A d on entry): with s = (w.r)/(w.w), mu += s d, r -= s w
@@ -699,6 +718,7 @@ struct bie_s {
   double* diag = nullptr;        // the operator's diagonal; A holds the rest as digits (k_matrix_digits)
   int* re = nullptr;             // row exponents
   int sms = 0;
+  bool cluster = false;          // the device can hold a cluster of k_arnoldi
   int ctas = 0, rows = 0;        // launch of k_gemv: one CTA per SM, rows of each
   double* gm = nullptr;          // H [(m+1) m], cs [m], sn [m], gv [m+2], y [m], hv [2(m+1)], scalars [8]
   double *ac = nullptr, *au = nullptr, *abv = nullptr;  // augmentation: c, u [2N], b [m]
@@ -798,12 +818,12 @@ extern "C" int bie_create(double alpha, double R, double A, int k, double phase,
   k_matrix_local<<<N, 128, 0, s>>>(B->np, alpha, L, B->star, nd, B->A);
   k_matrix_digits<<<B->n2, 256, 0, s>>>(B->n2, B->A, B->diag, B->re);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess ||
-      cudaFuncSetAttribute(k_arnoldi, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
       cudaFuncSetAttribute(k_gemv, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)gemv_smem(kMaxUnknowns, (kMaxUnknowns + B->ctas - 1) / B->ctas)) != cudaSuccess) {
     bie_free(B.release());
     return VP_ERR_CUDA;
   }
+  B->cluster = arnoldi_cluster_fits();
   *out = B.release();
   return VP_OK;
 }
@@ -880,7 +900,7 @@ extern "C" int bie_solve_aug(bie b, const double* g, double* mu, const double* d
     for (; j < jend; ++j) {
       const double* vj = b->V + (size_t)j * n;
       apply_operator(b, vj, b->w, s, ctl);
-      if (n <= kArnN && j < kArnCols) {
+      if (b->cluster && n <= kArnN && j < kArnCols) {
         k_arnoldi<<<kArnCtas, kArnThreads, 0, s>>>(n, j, M, tol, ctl, H, cs, sn, gv, b->w, b->V,
                                                    d ? b->ac : nullptr, b->abv);
         continue;
@@ -897,6 +917,7 @@ extern "C" int bie_solve_aug(bie b, const double* g, double* mu, const double* d
       k_gm_step<<<1, 1, 0, s>>>(j, M, tol, ctl, H, cs, sn, gv, hv, hv + M + 1, wn2 + 2);
       k_gm_scale<<<G, T, 0, s>>>(n, ctl, b->w, b->V + (size_t)(j + 1) * n);
     }
+    TRY(cudaGetLastError());  // a refused launch would leave `done` unset for every step to come
     TRY(cudaMemcpyAsync(b->hctl + slot, ctl, sizeof(GmresCtl), cudaMemcpyDeviceToHost, s));
     TRY(cudaEventRecord(b->ev[slot], s));
     if (jend > kGroup) {  // the group before this one
