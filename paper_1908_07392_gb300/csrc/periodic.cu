@@ -44,7 +44,9 @@ struct vp_periodic_s {
   int n = 0, logn = 0;
   int4* tw = nullptr;       // stage twiddles
   int4* wave = nullptr;     // k_x: mantissa digits, exponent
-  double* mult = nullptr;   // [n/2 + 1][n/2 + 1]: 1 / ((i^2 + j^2)(alpha^2 + |k|^2)), and 1 / alpha^2 at (0, 0)
+  double* mult = nullptr;   // [n/2 + 1][n/2 + 1]: 2^-mult_exp / ((i^2 + j^2)(alpha^2 + |k|^2)), and 2^-mult_exp / alpha^2
+                            // at (0, 0)
+  int mult_exp = 0;         // 128 where 1 / alpha^2 may be large: it meets spectra that are integers of up to 62 bits
   longlong2* z = nullptr;   // [kx][y] spectra along x, and two more columns of work space
   longlong2* a = nullptr;   // [y][kx] rows of A and D
   longlong2* d = nullptr;
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(Shape<LOGN>::threads, resident(Shape<LOGN>::th
 // n + 1 in place of the second one at kx = 0 and n / 2), every thread reading back what it wrote.
 template <int LOGN>
 __global__ void __launch_bounds__(Columns<LOGN>::threads, resident(Columns<LOGN>::threads))
-    k_columns(double two_pi_over_L, const double* __restrict__ mult, c64* Z, const int2* __restrict__ ez, c64* __restrict__ A,
+    k_columns(double two_pi_over_L, const double* __restrict__ mult, int mult_exp, c64* Z, const int2* __restrict__ ez, c64* __restrict__ A,
               c64* __restrict__ D, int* __restrict__ ea, int* __restrict__ ed, const int4* __restrict__ tw) {
   using S = Shape<LOGN>;
   using C = Columns<LOGN>;
@@ -422,7 +424,7 @@ __global__ void __launch_bounds__(Columns<LOGN>::threads, resident(Columns<LOGN>
     }
     if (C::turns == 2 && live) park[i + q * S::NT] = w[q];
   }
-  const int E1 = E;
+  const int E1 = E + mult_exp;
 
   // inverse transforms along y of u (d = 0) and k_y u (d = 1; the derivative is i times this, and the
   // Nyquist wavenumber carries none: its sine mode vanishes on the grid)
@@ -538,13 +540,13 @@ __global__ void __launch_bounds__(Shape<LOGN>::threads, resident(Shape<LOGN>::th
   }
 }
 
-__global__ void k_multiplier(int half, double alpha, double two_pi_over_L, double* mult) {
+__global__ void k_multiplier(int half, double alpha, double two_pi_over_L, double unit, double* mult) {
   const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const int w = half + 1;
   if (e >= (long long)w * w) return;
   const double i = (double)(e / w), j = (double)(e % w);
   const double r2 = i * i + j * j, k2 = two_pi_over_L * two_pi_over_L * r2;
-  mult[e] = r2 == 0.0 ? 1.0 / (alpha * alpha) : 1.0 / (r2 * (alpha * alpha + k2));
+  mult[e] = r2 == 0.0 ? unit / (alpha * alpha) : unit / (r2 * (alpha * alpha + k2));
 }
 
 // ------------------------------------------------------------------ twiddles (host)
@@ -639,7 +641,7 @@ int eval_size(const vp_periodic_s* P, const double* F, double* u, double* gradu,
   k_rows_forward<LOGN><<<S::n / S::rows, S::threads, smem_rows<LOGN>(), s>>>(F, P->z, P->ez, P->tw);
   TRY(cudaGetLastError());
   k_columns<LOGN><<<(S::n / 2 + C::cols) / C::cols, C::threads, smem_columns<LOGN>(), s>>>(
-      2.0 * kPi / P->side, P->mult, P->z, P->ez, P->a, P->d, P->ea, P->ed, P->tw);
+      2.0 * kPi / P->side, P->mult, P->mult_exp, P->z, P->ez, P->a, P->d, P->ea, P->ed, P->tw);
   TRY(cudaGetLastError());
   k_rows_inverse<LOGN><<<3 * (S::n / S::rows), S::threads, smem_rows<LOGN>(), s>>>(P->wave, P->a, P->d, P->ea, P->ed,
                                                                                     u, gradu, P->tw);
@@ -695,7 +697,9 @@ extern "C" int vp_periodic_create(double alpha, int n, double side, void* stream
     return fail(VP_ERR_OOM);
   const int rc = prepare_of(P->logn)();
   if (rc) return fail(rc);
-  k_multiplier<<<(unsigned)((hw * hw + 255) / 256), 256, 0, s>>>(n / 2, alpha, 2.0 * kPi / side, P->mult);
+  P->mult_exp = alpha < 1.0 ? 128 : 0;
+  k_multiplier<<<(unsigned)((hw * hw + 255) / 256), 256, 0, s>>>(n / 2, alpha, 2.0 * kPi / side, std::ldexp(1.0, -P->mult_exp),
+                                                                 P->mult);
   if (cudaMemcpyAsync(P->tw, tw.data(), tw.size() * sizeof(int4), cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaMemcpyAsync(P->wave, wave.data(), wave.size() * sizeof(int4), cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
