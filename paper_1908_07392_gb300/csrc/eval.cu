@@ -688,10 +688,12 @@ const double* table_ptr(const vp_tables_s* T, int t) {
 
 // Trees up to this many nodes launch their chain with programmatic dependent launch: CTAs that wait for the launch before
 // them keep near-field ones off their SMs, which costs more than the latency saved once the near field fills the chip.
-// Measured with / without: 64 leaves 93 / 111 us, 150,000 nodes 296 / 331 us, 10.5M nodes 7.02 / 6.78 ms; layers, whose
-// near part is small, 856 / 897 us (always on). Not under stream capture: in a graph of several trees the SMs that
-// waiting CTAs hold are another tree's (batch of four: 688 with, 641 us without).
-constexpr long long kPdlNodes = 300000;
+// Measured (Gaussian trees, p = 8 / 12 / 16, two channels) with over without: 150,000 nodes 0.96 / 0.87 / 0.86, 600,000
+// 0.96 / 0.89 / 0.96, 1.2M 1.00 / 0.99 / 0.96, 2.4M 1.05 / 1.05 / 1.04, 4.8M 1.03 / 1.04 / 1.05; one channel and uniform
+// trees cross at the same sizes, which differ in leaves by four. Layers, whose near part is small, 856 / 897 us (always
+// on). Not under stream capture: in a graph of several trees the SMs that waiting CTAs hold are another tree's
+// (batch of four: 688 with, 641 us without).
+constexpr long long kPdlNodes = 1500000;
 
 int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   const vp_tables_s* T = tr->T;
