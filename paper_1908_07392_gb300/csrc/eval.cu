@@ -1374,7 +1374,7 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
       if (rc) return rc;
     } else if (st.kind == 3) {
       const DevSlice& d = tr->slice_ops[st.index];
-      const int rc = launch_slice(bufs_c[d.buf], d.n, d.K, tr->sv[d.family], tr->se[d.family], s, pdl);
+      const int rc = launch_slice(bufs_c[d.buf], d.n, d.K, tr->sv[d.family], tr->se[d.family], s);
       if (rc) return rc;
       if (overlap && d.family == 0 && !near_started) {
         TRY(cudaEventRecord(tr->ev_src, s));
@@ -1393,7 +1393,7 @@ int run_steps(vp_tree_s* tr, const double* f, double* u, double* g, cudaStream_t
       a.dst_off = d.args.dst_off; a.ptr = d.args.ptr; a.slot = d.args.slot;
       a.S = bufs_c[d.src];
       a.u = u; a.g = g;
-      const int rc = launch_reduce_df(a, d.n_dst, s, pdl);
+      const int rc = launch_reduce_df(a, d.n_dst, s);
       if (rc) return rc;
     } else if (st.kind == 8) {
       const DevSum& d = tr->sums[st.index];

@@ -145,8 +145,6 @@ __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ X, lon
   const int L = 1 << lg_l, lane = threadIdx.x & 31, l = lane & (L - 1), warp = threadIdx.x >> 5;
   const long long v0 = (blockIdx.x * 8ll + warp) << (5 - lg_l), v = v0 + (lane >> lg_l);
   const bool ok = v < nvec;
-  pdl_trigger();
-  pdl_wait();
   const int count = (int)max(0ll, min(32ll >> lg_l, nvec - v0)) * K;  // at most 32 / L vectors of 8 L elements
   const double* src = X + v0 * K;
 #pragma unroll
@@ -882,8 +880,6 @@ __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, in
   const int d = blockIdx.x * (blockDim.x / per) + sub, r = 2 * t;
   const bool live = d < n_dst && r < a.M;
   const long long b = live ? a.ptr[d] : 0, e = live ? a.ptr[d + 1] : 0;
-  pdl_trigger();
-  pdl_wait();
   const float2* S = reinterpret_cast<const float2*>(a.S) + r;
   float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
   auto add = [&](float4 v) {
@@ -1148,13 +1144,13 @@ int launch_split_gemm(const SplitArgs& a, int n_tiles, cudaStream_t s, int engin
   return VP_OK;
 }
 
-int launch_slice(const double* X, long long nvec, int K, void* out, int* eb, cudaStream_t s, bool pdl) {
+int launch_slice(const double* X, long long nvec, int K, void* out, int* eb, cudaStream_t s) {
   if (nvec <= 0) return VP_OK;
   int lg_l = 2;  // lanes per vector: at least Kpad / 8, which is at most 32
   while ((8 << lg_l) < kpad(K)) ++lg_l;
   if (lg_l > 5) return VP_ERR_ARG;
-  TRY(launch(k_slice<kSplitSlices>, (unsigned)(((nvec << lg_l) + 255) / 256), 256, 0, s, pdl, X, nvec, K, kpad(K), lg_l,
-             (slice_t*)out, eb));
+  k_slice<kSplitSlices><<<(unsigned)(((nvec << lg_l) + 255) / 256), 256, 0, s>>>(X, nvec, K, kpad(K), lg_l, (slice_t*)out, eb);
+  TRY(cudaGetLastError());
   return VP_OK;
 }
 
@@ -1171,7 +1167,7 @@ int launch_sum_slice(int C, int nseg, long long n, const long long* ptr, const l
   return VP_OK;
 }
 
-int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s, bool pdl) {
+int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s) {
   if (n_dst <= 0) return VP_OK;
   const int pairs = (a.M + 1) / 2;
   if (pairs > 512) return VP_ERR_ARG;  // 3 p^2 <= 768 rows
@@ -1180,7 +1176,8 @@ int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s, bool pdl)
   const unsigned blocks = (unsigned)((n_dst + threads / per - 1) / (threads / per));
   auto even = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   // n even: a pair of rows lies in one field, and destinations and N are even too
-  TRY(launch(k_reduce_df, blocks, threads, 0, s, pdl, a, n_dst, per, a.n % 2 == 0 && even(a.u) && even(a.g)));
+  k_reduce_df<<<blocks, threads, 0, s>>>(a, n_dst, per, a.n % 2 == 0 && even(a.u) && even(a.g));
+  TRY(cudaGetLastError());
   return VP_OK;
 }
 

@@ -90,8 +90,8 @@ int read_split_error(int* flag);
 // Run a kernel whose bounded wait on an mbarrier nothing arrives at gives up after `budget` clocks.
 int selftest_wait(long long budget, cudaStream_t s);
 // nvec consecutive vectors of K elements into digits and exponents (k_slice).
-int launch_slice(const double* X, long long nvec, int K, void* out, int* eb, cudaStream_t s, bool pdl = false);
-int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s, bool pdl = false);
+int launch_slice(const double* X, long long nvec, int K, void* out, int* eb, cudaStream_t s);
+int launch_reduce_df(const DFReduceArgs& a, int n_dst, cudaStream_t s);
 // Sums of double-float slots sliced in place of being stored (k_sum_slice): n vectors of nseg segments of C elements.
 int launch_sum_slice(int C, int nseg, long long n, const long long* ptr, const long long* slot, const long long* vid,
                      const void* slots, void* out, int* eb, cudaStream_t s, bool pdl = false);
