@@ -25,7 +25,10 @@ typedef struct bie_s* bie;
 
 /*
  * bie_create -- nodes and the dense Nystrom matrix (2N x 2N, on the device) for alpha > 0: computed in FP64 and kept as
- * 63-bit integers with one exponent per row (rounding 2^-63 of a row's largest entry), the diagonal apart in FP64.
+ * 63-bit integers with one exponent per row (rounding 2^-63 of a row's largest entry), the diagonal apart in FP64. An
+ * apply takes the vector as 72-bit integers (rounding 2^-72 of its largest component): entries below 2^-9 of their row's
+ * largest and components below 2^-18 of the vector's keep fewer than FP64's bits, and the error of an apply is about
+ * half of FP64's.
  * Entries from the target's own panel and its two neighbours come from a graded local quadrature
  * of the kernel against the panel's Lagrange basis (the kernel's r log r terms); the rest are plain
  * Gauss-Legendre. max_krylov (1..1000) sizes the GMRES work space. Synchronises `stream`.

@@ -95,9 +95,13 @@ enum {
  *             contraction -- near tables, source-to-multipole, multipole-to-
  *             multipole, multipole-to-local, source-to-local, local-to-local,
  *             local-to-target, multipole-to-target -- on the tensor cores from
- *             exact 8-bit bf16 slices of the FP64 operands, folded in
- *             double-float; the kernel values and the level scaling of the
- *             operators are computed in FP64).
+ *             exact 8-bit bf16 slices of the FP64 operands: 48 bits of a
+ *             row's or a vector's largest element. Contributions are
+ *             double-float (two fp32: 48 bits, exponents of fp32, so sources
+ *             scaled below about 2^-60 lose low bits and results above
+ *             3e38 overflow); those of an expansion are summed in three fp32
+ *             words, those of an output in two. The kernel values and the
+ *             level scaling of the operators are computed in FP64).
  *  stream     stream for the build kernels; the call synchronises it before
  *             returning.
  *  out        receives the handle; free with vp_tables_free.
@@ -386,7 +390,8 @@ int vp_eval_static(vp_tree tree, const double* f, double* u, double* gradu, void
  *  4  tcgen05 on transposed tiles: the tile's 128 columns are the MMA's rows and the operator's rows
  *     its N (rounded up to 96 or 128), so operators of at most 128 rows (the 81-row multipole and
  *     local operators) fill every tensor-memory lane; launches with taller operators run on engine 1.
- * All compute the same exact slice sums. Until a tree is tuned its launches use engines 1, 3 and 4, by rows and number
+ * All compute the same slice sums, engines 0 to 3 to the same bits; engine 4 rounds the sum of the smallest
+ * products (below 2^-24 of the result) in another order. Until a tree is tuned its launches use engines 1, 3 and 4, by rows and number
  * of tiles. vp_tree_set_engine sets one engine for every launch of
  * the tree (VP_ERR_ARG for other values). vp_autotune times each split-precision launch of one
  * evaluation of `f` with every engine (tile shape) on `stream`, keeps the fastest per launch shape,

@@ -61,7 +61,8 @@ struct GemmArgs {
 // small as they need to be for little work on padding: rows are skipped in groups of 8 and columns in groups of 4
 // past the tile's own, and K ends where it ends (81-row operators run 88 of them, not 128, and groups of a few
 // columns only those). Measured (583-leaf adaptive tree, p = 16, both channels): near launch 3,343 -> 1,720 us =
-// 1.14 TFLOP/s, 0.91 of the pipe; M2L 973 -> 416 us (64 x 64 tiles computed whole).
+// 1.14 TFLOP/s, 0.91 of the pipe, M2L 973 -> 416 us (64 x 64 tiles computed whole); the 10.5M-node star's near launch,
+// whose waves are many, 0.997 of the pipe.
 constexpr int kBM = 32, kBN = 32, kBK = 16, kGemmThreads = 128;
 // Launches of fewer tiles (16 per SM of the 152) leave SMs idle or uneven: they run on tiles of 8 x 4
 // (k_gemm_small_f64). Measured with the line at 608, 1216 and 2432 tiles: uniform depth 4, p = 11, 355, 311 and 311 us;
@@ -1690,7 +1691,6 @@ int time_split_launches(vp_tree_s* tr, const double* f, double* u, double* g, in
     DevSplit d = tr->splits[k];
     d.engine = engine;
     SplitArgs a = split_args(tr, d, bufs);
-    // accumulating outputs are only timed (their values are rebuilt by the next full evaluation)
     if (cudaEventRecord(ev[2 * k], s) != cudaSuccess) rc = VP_ERR_CUDA;
     if (rc == VP_OK) rc = launch_split_gemm(a, d.n_tiles[engine], s, engine);
     if (rc == VP_OK && cudaEventRecord(ev[2 * k + 1], s) != cudaSuccess) rc = VP_ERR_CUDA;

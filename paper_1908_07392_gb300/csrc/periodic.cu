@@ -27,8 +27,8 @@
 // pass), 2048^2 0.564 ms (3.6), 512^2 56 us (about 250). The error against long double is 0.2 to 0.9 of the
 // FP64 form's in the 2-norm (32^2 .. 2048^2; white noise, few modes, point forces). What bounds it: 2048^2 runs
 // at 2 to 2.4 instructions per clock and SM of 4, the integer pipe half busy, the rest latency (about 330
-// instructions per point and transform), 4096^2 at 1.4 with one CTA of k_columns per SM (registers); 155 bytes per
-// point of DRAM traffic would take 0.1 ms.
+// instructions per point and transform), 4096^2 at 1.4 with one CTA of k_columns per SM (registers, of which it
+// spills some); 160 bytes per point at the copy rate would take 0.10 ms at 2048^2, 0.40 at 4096^2.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -183,8 +183,9 @@ struct Columns {
 };
 
 // CTAs per SM the compiler leaves registers for: 64 a thread where CTAs are large and throughput counts, 128
-// (no spills) where they are small and a thread's own speed does (512^2: 64, 80 and 128 registers 64.5, 58.4 and 56.3
-// us; at 1024^2 more than 64 are slower, 189 against 172 us).
+// where they are small and a thread's own speed does (512^2: 64, 80 and 128 registers 64.5, 58.4 and 56.3
+// us; at 1024^2 more than 64 are slower, 189 against 172 us). k_columns spills 460 to 604 bytes a thread at 64 registers
+// (1024^2 and up) and 20 at 512^2; the row kernels and the smaller columns spill nothing.
 constexpr int resident(int threads) { return (threads >= 256 ? 1024 : 512) / threads; }
 
 enum { RED_OR, RED_MAX };

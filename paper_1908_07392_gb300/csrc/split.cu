@@ -18,8 +18,11 @@
 //     accumulator whose rounding is below 2^-48 of the result;
 //   * the four sums are added in double-float (two fp32) and scaled by
 //     2^(ea[r] + eb) exactly. Products with i + j > S - 1 are dropped.
-// Two engines run the same arithmetic: warp-level mma.sync (m16n8k16 bf16),
-// and tcgen05.mma with the accumulators in tensor memory.
+// Contributions are double-float slots (exact but for FP32's exponent range, as the outputs' are); those of an
+// expansion are summed in three fp32 words (fsum.h).
+// Five engines run the same arithmetic: warp-level mma.sync (m16n8k16 bf16) on tiles of two sizes, and tcgen05.mma with
+// the accumulators in tensor memory on tiles of 128 x 128, 128 x 64 and transposed. All but the transposed one give the same
+// bits; that one adds the tail's products in another order.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -134,10 +137,10 @@ __device__ inline void store_digits(const unsigned long long (&t)[8], unsigned n
 //
 // L lanes per vector (a power of two, L >= Kpad / 8), a lane taking 8 consecutive elements: they are read once and
 // kept for the digits, and a slice of them is one 16-byte store (2-byte stores, six per element, and a second
-// read of the vector took 571 us an evaluation of the full-size star, now 459). A warp's vectors are consecutive, so
+// read of the vector took 79 us for the star's leaf sources). A warp's vectors are consecutive, so
 // they are read in order and dealt out through shared memory: X may be page-locked host memory, which lanes reading
 // their own 64 bytes piece by piece took 324 us for 4.2M elements to fetch (172 in order; 27 and 30 us from the device).
-// Measured: the star's leaf sources (40,897 vectors of 256) 79 -> 52 us = 4.0 TB/s.
+// Measured: the star's leaf sources (40,897 vectors of 256) 54.5 us = 3.8 TB/s.
 template <int S>
 __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ X, long long nvec, int K, int Kpad, int lg_l,
                                                slice_t* __restrict__ out, int* __restrict__ eb) {
@@ -931,9 +934,9 @@ __global__ void __launch_bounds__(512) k_reduce_df(DFReduceArgs a, int n_dst, in
 //
 // One warp per vector: lane t sums elements t, t + 32, .. (coalesced reads, kSumFlight slots in flight), the sums
 // pass through shared memory, and lanes of 8 consecutive elements form the digits. Measured: full-size star, locals of
-// 40,892 leaves from 1.17 GB of slots 252 us = 4.6 TB/s; all of its sums 661 us in place of 278 us of reductions into
-// FP64 expansions and about 400 us of slicing, and the upward and downward contractions, which added to FP64 values in
-// memory, 335 us instead of 880.
+// 40,892 leaves from 1.17 GB of slots 233 us = 5.0 TB/s (252 with two-word sums and FP64 conversions); all of its sums
+// 596 us in place of 278 us of reductions into FP64 expansions and about 400 us of slicing, and the upward and downward
+// contractions, which added to FP64 values in memory, 323 us instead of 880.
 constexpr int kSumWarps = 4, kSumFlight = 4;
 
 template <int S, int NSEG, int QC>  // QC: elements of a segment per lane
