@@ -98,7 +98,7 @@ enum {
  *             exact 8-bit bf16 slices of the FP64 operands: 48 bits of a
  *             row's or a vector's largest element. Contributions are
  *             double-float (two fp32: 48 bits, exponents of fp32, so sources
- *             scaled below about 2^-60 lose low bits and results above
+ *             scaled below about 2^-45 lose low bits and results above
  *             3e38 overflow); those of an expansion are summed in three fp32
  *             words, those of an output in two. The kernel values and the
  *             level scaling of the operators are computed in FP64).
