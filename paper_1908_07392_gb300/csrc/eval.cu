@@ -383,11 +383,19 @@ struct DevSum {
   long long n;
   const long long *ptr, *slot, *vid;
 };
+struct SlotRun {  // slots first, first + step, .. (n of them)
+  long long first = 0, step = 0;
+  int n = 0;
+};
 struct HostSum {
   int family = 0, buf = 0, nseg = 1;
   std::vector<long long> ptr{0}, slot, vid;
   void segment(const std::vector<long long>& slots) {
     slot.insert(slot.end(), slots.begin(), slots.end());
+    ptr.push_back((long long)slot.size());
+  }
+  void segment(const SlotRun& r) {
+    for (int k = 0; k < r.n; ++k) slot.push_back(r.first + k * r.step);
     ptr.push_back((long long)slot.size());
   }
 };
@@ -496,6 +504,8 @@ int upload_gemm(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
                    [](const HostGemm::Entry& x, const HostGemm::Entry& y) { return x.a < y.a; });
   std::vector<long long> a_off, src_off, dst_off;
   std::vector<Tile> tiles, groups;
+  src_off.reserve(g.entries.size());
+  dst_off.reserve(g.entries.size());
   size_t i = 0;
   while (i < g.entries.size()) {
     size_t j = i;
@@ -512,6 +522,9 @@ int upload_gemm(vp_tree_s* tr, HostGemm& g, cudaStream_t s) {
   for (const Tile& t : groups) n_big += (long long)((g.M + kBM - 1) / kBM) * ((t.ncol + kBN - 1) / kBN);
   d.small = n_big < kSmallTiles;
   const int bm = d.small ? kBMs : kBM, bn = d.small ? kBNs : kBN;
+  size_t n_tiles = 0;
+  for (const Tile& t : groups) n_tiles += (size_t)((g.M + bm - 1) / bm) * ((t.ncol + bn - 1) / bn);
+  tiles.reserve(n_tiles);
   for (const Tile& t : groups)
     for (int m0 = 0; m0 < g.M; m0 += bm)
       for (int c0 = 0; c0 < t.ncol; c0 += bn) tiles.push_back({t.group, m0, t.col0 + c0, std::min(bn, t.ncol - c0)});
@@ -761,7 +774,7 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
   // summed and sliced level by level; in FP64 BUF_MP and BUF_LOC hold the expansions themselves
   const int Es = (E + 3) & ~3;
   long long nup = 0;
-  std::vector<std::vector<long long>> upl(split ? (size_t)NB * nch : 0);
+  std::vector<SlotRun> upl(split ? (size_t)NB * nch : 0);
   for (long long i = 0; i < NB; ++i) {
     const Box& b = B[i];
     if (b.leaf < 0 || b.level < 2) continue;
@@ -770,7 +783,7 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
     l2t.entries.push_back({(long long)(b.level * T->l2t_stride_lvl()), i * E, slot * Us});
     s2m.entries.push_back({(long long)(b.level * T->s2m_stride_lvl()), (long long)b.leaf * n, split ? nup : i * E});
     if (!split) continue;
-    for (int ch = 0; ch < nch; ++ch) upl[i * nch + ch].push_back(nup + ch * C);
+    for (int ch = 0; ch < nch; ++ch) upl[i * nch + ch] = {nup + ch * C, 0, 1};
     nup += Es;
   }
   std::vector<HostGemm> up(split ? P.max_level + 1 : 0), down(up.size());
@@ -785,12 +798,12 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
     for (long long i = 0; i < NB; ++i) {
       const int l = B[i].level;
       for (int ch = 0; ch < nch; ++ch) {
-        if (B[i].leaf < 0 && l >= 2 && (ch || kact(l)))
-          for (int q = 0; q < 4; ++q, nup += Cs) {
+        if (B[i].leaf < 0 && l >= 2 && (ch || kact(l))) {
+          upl[i * nch + ch] = {nup, Cs, 4};
+          for (int q = 0; q < 4; ++q, nup += Cs)
             up[l].entries.push_back({(q * part + (long long)l * nch + ch) * mat, (long long)(B[i].child0 + q) * E + ch * C, nup,
                                      (long long)(B[i].child0 + q) * nch + ch});
-            upl[i * nch + ch].push_back(nup);
-          }
+        }
         if (l >= 3 && (ch || kact(l - 1))) {
           const int par = B[i].parent, q = (int)(i - B[par].child0);
           const long long slot = nls++;
@@ -850,7 +863,8 @@ int build_tree(vp_tree_s* tr, const TreePlan& P, cudaStream_t s) {
       for (long long i = lvl[l]; i < lvl[l + 1]; ++i)
         for (int ch = 0; ch < nch; ++ch) {
           if (!upward && (B[i].leaf >= 0 || !(ch || kact(l)))) continue;
-          h.segment((upward ? upl : lsl)[i * nch + ch]);
+          if (upward) h.segment(upl[i * nch + ch]);
+          else h.segment(lsl[i * nch + ch]);
           h.vid.push_back(i * nch + ch);
         }
       return upload_sum(tr, h, s);
@@ -1017,7 +1031,7 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
   const bool split = T->precision == VP_PREC_SPLIT;
   const int Es = (E + 3) & ~3;
   long long nup = 0;
-  std::vector<std::vector<long long>> upl(split ? (size_t)NC * NB * nch : 0);
+  std::vector<SlotRun> upl(split ? (size_t)NC * NB * nch : 0);
   std::vector<PtInst> ps2m, ps2l, pnear;
   for (long long i = 0; i < NB; ++i) {
     const Box& b = B[i];
@@ -1030,9 +1044,7 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
     if (!split) continue;
     // a slot per component, then those of the remainders: the sources' FP64 sums enter whole
     for (int a = 0; a < NC; ++a)
-      for (int ch = 0; ch < nch; ++ch)
-        for (int part = 0; part < 2; ++part)
-          upl[(size_t)(a * NB + i) * nch + ch].push_back(nup + (part * NC + a) * Es + ch * C);
+      for (int ch = 0; ch < nch; ++ch) upl[(size_t)(a * NB + i) * nch + ch] = {nup + a * Es + ch * C, (long long)NC * Es, 2};
     nup += 2 * NC * Es;
   }
   HostGemm m2l, l2t, m2t;
@@ -1118,7 +1130,8 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
               if (!has[c]) continue;
               up[l].entries.push_back({(q * part + (long long)l * nch + ch) * mat, off(a, c) + ch * C, nup,
                                        (a * NB + c) * nch + ch});
-              upl[(size_t)(a * NB + i) * nch + ch].push_back(nup);
+              SlotRun& r = upl[(size_t)(a * NB + i) * nch + ch];
+              if (r.n++ == 0) r = {nup, Cs, 1};
               nup += Cs;
             }
           if (l >= 3 && (ch || kact(l - 1))) {
@@ -1168,7 +1181,8 @@ int build_layer(vp_tree_s* tr, const TreePlan& P, const LayerBins& bins, const P
         for (long long i : at[l])
           for (int ch = 0; ch < nch; ++ch) {
             if (upward ? !has[i] : (B[i].leaf >= 0 || !(ch || kact(l)))) continue;
-            h.segment((upward ? upl : lsl)[(size_t)(a * NB + i) * nch + ch]);
+            if (upward) h.segment(upl[(size_t)(a * NB + i) * nch + ch]);
+            else h.segment(lsl[(size_t)(a * NB + i) * nch + ch]);
             h.vid.push_back((a * NB + i) * nch + ch);
           }
       return upload_sum(tr, h, s);
