@@ -661,31 +661,35 @@ extern "C" int ws_create(int in_ch, int width, int out_ch, int n_layers, int ksi
   if ((rc = walloc(w.get(), &w->d0, (size_t)max_batch * maxc * n)) ||
       (rc = walloc(w.get(), &w->d1, (size_t)max_batch * maxc * n)))
     return fail(rc);
-  size_t parts = 0;
-  w->wf.assign(n_layers, nullptr);
-  w->wb.assign(n_layers, nullptr);
+  // the layouts of all layers in one piece, zero where they are padded; the part sums
+  size_t parts = 0, lay = 0;
+  std::vector<Layer> layers(n_layers);
   for (int l = 0; l < n_layers; ++l) {
-    const size_t nf = (size_t)w->C[l] * ksize * pad4(w->C[l + 1]), nb = (size_t)w->C[l + 1] * ksize * pad4(w->C[l]);
-    if ((rc = walloc(w.get(), &w->wf[l], nf)) || (rc = walloc(w.get(), &w->wb[l], nb))) return fail(rc);
-    if (cudaMemsetAsync(w->wf[l], 0, nf * sizeof(float), s) != cudaSuccess ||
-        cudaMemsetAsync(w->wb[l], 0, nb * sizeof(float), s) != cudaSuccess)
-      return fail(VP_ERR_CUDA);
-    parts = std::max(parts, part_floats(wgrad_tiles(w->C[l], w->C[l + 1], ksize), wgrad_segs(n, max_batch)));
+    const int cin = w->C[l], cout = w->C[l + 1];
+    lay += (size_t)cin * ksize * pad4(cout) + (size_t)cout * ksize * pad4(cin);
+    parts = std::max(parts, part_floats(wgrad_tiles(cin, cout, ksize), wgrad_segs(n, max_batch)));
   }
   w->part_count = parts;
-  if ((rc = walloc(w.get(), &w->wparts, parts)) || (rc = prepare_of(ksize)())) return fail(rc);
-  std::vector<Layer> layers(n_layers);
-  for (int l = 0; l < n_layers; ++l) layers[l] = {w->woff[l], w->boff[l], w->C[l], w->C[l + 1], w->wf[l], w->wb[l]};
+  float* at = nullptr;
+  if ((rc = walloc(w.get(), &at, lay)) || (rc = walloc(w.get(), &w->wparts, parts)) || (rc = prepare_of(ksize)()))
+    return fail(rc);
+  if (cudaMemsetAsync(at, 0, lay * sizeof(float), s) != cudaSuccess) return fail(VP_ERR_CUDA);
+  for (int l = 0; l < n_layers; ++l) {
+    const int cin = w->C[l], cout = w->C[l + 1];
+    float* wb = at + (size_t)cin * ksize * pad4(cout);
+    layers[l] = {w->woff[l], w->boff[l], cin, cout, at, wb};
+    w->wf.push_back(at);
+    w->wb.push_back(wb);
+    at = wb + (size_t)cout * ksize * pad4(cin);
+  }
   {
-    void *q = nullptr, *d = nullptr;
-    if (cudaMalloc(&q, 256 * sizeof(double)) != cudaSuccess) return fail(VP_ERR_OOM);
+    void* q = nullptr;
+    const size_t sums = 256 * sizeof(double), bytes = layers.size() * sizeof(Layer);
+    if (cudaMalloc(&q, sums + bytes) != cudaSuccess) return fail(VP_ERR_OOM);
     w->allocs.push_back(q);
     w->part = static_cast<double*>(q);
-    if (cudaMalloc(&d, layers.size() * sizeof(Layer)) != cudaSuccess) return fail(VP_ERR_OOM);
-    w->allocs.push_back(d);
-    w->layers = static_cast<Layer*>(d);
-    if (cudaMemcpyAsync(d, layers.data(), layers.size() * sizeof(Layer), cudaMemcpyHostToDevice, s) != cudaSuccess)
-      return fail(VP_ERR_CUDA);
+    w->layers = reinterpret_cast<Layer*>(w->part + 256);
+    if (cudaMemcpyAsync(w->layers, layers.data(), bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return fail(VP_ERR_CUDA);
   }
   // initial parameters: uniform in +-1/sqrt(fan_in) from a seeded splitmix64 stream
   std::vector<float> host(off);
